@@ -18,7 +18,8 @@
 namespace fastged {
 
 constexpr int kMaxWords = 16;       // 1024 vertices
-constexpr int kHistMax = 32;        // PED histogram buckets (one per lane)
+constexpr int kHistMax = 32;        // PEDs a kept list may span (one lane per PED ranks them)
+constexpr int kHistRow = 128;       // counters of a warp's PED histogram row
 constexpr int kMaxB = 8;            // edge-label bit-planes (labels 0..255)
 constexpr int kMaxWarps = 16;       // 512 threads per CTA
 constexpr int kMaxClusterWarps = 256; // 16 CTAs of 512 threads
@@ -38,7 +39,7 @@ struct GraphMeta {
 enum Region : int {
     RG_HIST = 0, RG_ALPHA2, RG_A2T, RG_L2T, RG_SBASE, RG_PED0, RG_PED1, RG_SEL, RG_SELPED,
     RG_KLIST, RG_KPED, RG_NOFF, RG_NBR, RG_IMG0, RG_IMG1, RG_P, RG_PL,
-    RG_CAND, RG_MAP0, RG_MAP1, RG_IMGL, RG_CROW,
+    RG_SCORE, RG_MAP0, RG_MAP1, RG_IMGL, RG_CROW, RG_ACT, RG_ALL, RG_REC, RG_CHIST,
     RG_COUNT
 };
 
@@ -52,16 +53,15 @@ struct Layout {
     int32_t n1max, n2max;      // largest graphs of the class
     int32_t n2s;               // row stride (elements) of the transposed g2 tables
     int32_t mrow;              // bytes per stored vertex map
-    int32_t fs;                // successors per node at most (n2max + 1)
     int32_t word_bytes;        // 4 or 8: bytes per bitset word
     int32_t B;                 // edge-label planes
-    int32_t pk;                // 1: successors packed as PED << 16 | slot << jbits | j
     int64_t smem_bytes;        // dynamic shared memory per CTA
     int64_t slice_bytes;       // global scratch bytes per team (CTA or cluster)
     int64_t team_off;          // cluster teams: offset of the team scalars in the slice
     // cluster teams: per-CTA tables that did not fit shared memory live in a block of the
     // slice per CTA (at cta_off + cluster rank * cta_bytes; their off[] is inside the block)
     uint32_t cta_mask;
+    int64_t jm_off;            // single-word teams: one-hot vertex bits inside RG_REC
     int64_t cta_off, cta_bytes;
     int64_t rsize[RG_COUNT];   // bytes of every region (bounds-checked builds check against it)
 };
@@ -92,6 +92,13 @@ enum WarpRegion : int {
 constexpr int warp_rec_bytes(bool w32, int npl)
 {
     return ((w32 ? 4 : 8) * (1 + npl) + 4 + 15) / 16 * 16;
+}
+
+// bytes of one column record of the single-word teams (ColRec): adjacency word, label planes
+// (at least one slot) and the 32-bit cost-row entry
+constexpr int col_rec_bytes(bool w32, int npl)
+{
+    return ((w32 ? 4 : 8) * (1 + (npl > 0 ? npl : 1)) + 4 + 15) / 16 * 16;
 }
 
 struct WarpLayout {

@@ -407,7 +407,6 @@ fastged_options fastged::default_options()
 void fastged::plan_layout(ClassPlan &cp, int B, int block, size_t budget)
 {
     Layout &L = cp.lay;
-    const int NW = (block / 32) * cp.cluster;   // warps of the whole team
     const int W = cp.W;
     const size_t msz = cp.wide ? 2 : 1;
     const size_t wb = cp.w32 ? 4 : 8;
@@ -416,16 +415,22 @@ void fastged::plan_layout(ClassPlan &cp, int B, int block, size_t budget)
     L.n2max = cp.n2max;
     L.n2s = (int)align_up((size_t)std::max(cp.n2max, 1) + 1, 4);
     L.mrow = (int)align_up((size_t)std::max(cp.n1max, 1) * msz, 16);
-    L.fs = cp.n2max + 1;
     L.word_bytes = (int)wb;
     L.B = B;
     size_t sz[RG_COUNT];
     const size_t km = (size_t)cp.kmax;
-    const size_t ncand = km * ((size_t)cp.n2max + 1);
     // node slots a CTA prepares: all of them, or its share of a cluster team
     const size_t kl = cp.cluster > 1 ? (km + cp.cluster - 1) / cp.cluster + 1 : km;
     L.kloc = (int32_t)kl;
-    sz[RG_HIST] = (size_t)kHistMax * NW * 4;
+    sz[RG_HIST] = (size_t)(block / 32 + 1) * kHistRow * 4;   // a row per warp, and the totals
+    sz[RG_ACT] = (size_t)L.n2s * 2;
+    sz[RG_ALL] = (size_t)W * wb;
+    // single-word teams: a record and a one-hot word per active column, in whole quads, an odd
+    // number of them
+    const size_t cols = W == 1 ? align_up((size_t)cp.n2max + 1, 4) + 4 : 0;
+    L.jm_off = (int64_t)(cols * (size_t)col_rec_bytes(cp.w32, label_instance(B)));
+    sz[RG_REC] = (size_t)L.jm_off + cols * wb;
+    sz[RG_CHIST] = cp.cluster > 1 ? (size_t)cp.cluster * kHistRow * 4 : 0;
     sz[RG_ALPHA2] = (size_t)L.n2s * 4;
     sz[RG_CROW] = (size_t)2 * L.n2s * 4;
     sz[RG_A2T] = (size_t)W * L.n2s * wb;
@@ -444,30 +449,30 @@ void fastged::plan_layout(ClassPlan &cp, int B, int block, size_t budget)
     sz[RG_P] = kl * W * wb;
     sz[RG_PL] = (size_t)B * kl * W * wb;
     sz[RG_IMGL] = cp.cluster > 1 ? kl * W * wb : 0;
-    // single-word classes pack the successor ids into the PED entries
-    // one entry per successor: 32 bits when packed, else 64 (PED, parent slot, j)
-    const bool packed = cp.pk && cp.cluster == 1;
-    L.pk = packed ? 1 : 0;
-    sz[RG_CAND] = ncand * (packed ? 4 : 8);
+    // one byte per successor of the CTA's nodes
+    sz[RG_SCORE] = kl * (W == 1 ? ((cols / 4 - 1) | 1) * 4 : (size_t)cp.n2max + 1);
     sz[RG_MAP0] = km * L.mrow;
     sz[RG_MAP1] = km * L.mrow;
     // shared memory is filled in order of access frequency; the rest goes to global scratch
-    static const int prio[RG_COUNT] = {RG_HIST, RG_CROW, RG_ALPHA2, RG_SBASE, RG_PED0, RG_PED1,
-                                       RG_SEL, RG_SELPED, RG_KLIST, RG_KPED, RG_NOFF,
-                                       RG_A2T, RG_L2T, RG_IMG0, RG_IMG1, RG_P, RG_PL,
-                                       RG_CAND, RG_NBR, RG_MAP0, RG_MAP1, RG_IMGL};
+    // (RG_HIST, RG_ACT, RG_ALL and RG_REC come first in both orders: the kernels rely on them being
+    // there)
+    static const int prio[RG_COUNT] = {RG_HIST, RG_ACT, RG_ALL, RG_REC, RG_CROW, RG_ALPHA2, RG_SBASE,
+                                       RG_PED0, RG_PED1, RG_SEL, RG_SELPED, RG_KLIST, RG_KPED,
+                                       RG_NOFF, RG_A2T, RG_L2T, RG_IMG0, RG_IMG1, RG_P, RG_PL,
+                                       RG_SCORE, RG_NBR, RG_MAP0, RG_MAP1, RG_IMGL, RG_CHIST};
     // cluster teams: the per-CTA tables the CTA writes (P, PL, sbase, staged Img) must be in
     // shared memory, so they come first
-    static const int prio_cl[RG_COUNT] = {RG_SBASE, RG_P, RG_PL, RG_IMGL, RG_CROW, RG_ALPHA2,
-                                          RG_NOFF,
-                                          RG_A2T, RG_L2T, RG_NBR, RG_HIST, RG_PED0, RG_PED1,
-                                          RG_SEL, RG_SELPED, RG_KLIST, RG_KPED, RG_IMG0,
-                                          RG_IMG1, RG_CAND, RG_MAP0, RG_MAP1};
+    static const int prio_cl[RG_COUNT] = {RG_HIST, RG_ACT, RG_ALL, RG_REC, RG_SBASE, RG_P, RG_PL,
+                                          RG_IMGL, RG_CROW, RG_ALPHA2, RG_NOFF, RG_A2T, RG_L2T,
+                                          RG_SCORE, RG_NBR, RG_CHIST, RG_PED0, RG_PED1, RG_SEL,
+                                          RG_SELPED, RG_KLIST, RG_KPED, RG_IMG0, RG_IMG1,
+                                          RG_MAP0, RG_MAP1};
     // a cluster team shares only global memory: its CTAs keep private shared-memory copies
     // of the read-only target-graph tables and neighbour lists, everything else is global
     auto cta_local = [](int r) {
         return r == RG_ALPHA2 || r == RG_A2T || r == RG_L2T || r == RG_NOFF || r == RG_NBR ||
-               r == RG_P || r == RG_PL || r == RG_SBASE || r == RG_IMGL || r == RG_CROW;
+               r == RG_P || r == RG_PL || r == RG_SBASE || r == RG_IMGL || r == RG_CROW ||
+               r == RG_HIST || r == RG_ACT || r == RG_ALL || r == RG_REC || r == RG_SCORE;
     };
     for (int r = 0; r < RG_COUNT; ++r) L.rsize[r] = (int64_t)align_up(sz[r], 16);
 #ifdef FASTGED_BOUNDS_CHECK
@@ -505,6 +510,15 @@ void fastged::plan_layout(ClassPlan &cp, int B, int block, size_t budget)
     }
     L.smem_bytes = (int64_t)s_used;
     L.slice_bytes = (int64_t)align_up(g_used, 256);
+}
+
+bool fastged::layout_in_smem(const Layout &L)
+{
+    for (int r = 0; r < RG_COUNT; ++r)
+        if (r != RG_NBR && r != RG_MAP0 && r != RG_MAP1 && L.rsize[r] > 0 &&
+            !((L.smem_mask >> r) & 1u))
+            return false;
+    return true;
 }
 
 size_t fastged::plan_warp_layout(ClassPlan &cp, int B, bool gmap)
@@ -552,7 +566,6 @@ size_t fastged::plan_warp_layout(ClassPlan &cp, int B, bool gmap)
     cp.lay.n1max = cp.n1max;
     cp.lay.n2max = cp.n2max;
     cp.lay.word_bytes = (int32_t)wb;
-    cp.lay.pk = 1;
     return sh;
 }
 
@@ -778,7 +791,7 @@ static int tune_class(fastged_handle *h, ClassPlan &cp, int B, int forced_block,
         budget = std::min(max_dyn, per_sm / 2 - stat);    // keep two teams per SM
     }
     plan_layout(cp, B, block, budget);
-    cp.all_smem = cp.lay.slice_bytes == 0 && kbest_has_smem_variant(cp.W, cp.wide, cp.w32);
+    cp.all_smem = layout_in_smem(cp.lay) && kbest_has_smem_variant(cp.W, cp.wide, cp.w32);
     int occ = 0;
     cudaError_t e = kbest_occupancy(cp.W, cp.wide, cp.w32, cp.all_smem, label_instance(B), block,
                                     (size_t)cp.lay.smem_bytes, &occ);
@@ -1006,9 +1019,8 @@ int fastged::flatten(fastged_handle *h, const fastged_pair_list *pl, int32_t K,
                                     (long long)g2.m * c.e_ins;
             if (bound >= (long long)INT32_MAX) { ferr.put(p, where() + ": costs can overflow int32"); break; }
             int W = words_class(g2.n);
-            // packing (PED, parent slot, j) into 32 bits needs every PED below 2^16 (PEDs
-            // never count vertex insertions, and at most the g2 edges among mapped vertices)
-            // and K within the slot field
+            // see packable(); PEDs never count vertex insertions, and at most the g2 edges
+            // among mapped vertices
             const long long ped_bound = (long long)g1.n * std::max(c.v_sub, c.v_del) +
                                         (long long)g1.m * std::max(c.e_sub, c.e_del) +
                                         (long long)g2.m * c.e_ins;

@@ -81,6 +81,9 @@ int set_error(int code, const char *msg);
 // splits a team's working set into shared-memory and global-scratch regions (budget bytes of
 // shared memory, filled in order of access frequency)
 void plan_layout(ClassPlan &cp, int B, int block, size_t budget);
+// true when every region but the neighbour lists and the vertex maps is in shared memory (the
+// kernels' all-shared-memory variant)
+bool layout_in_smem(const Layout &L);
 // lays out one warp's working set for a one-warp class; gmap puts the vertex maps in global
 // scratch. Returns the shared-memory bytes per warp.
 size_t plan_warp_layout(ClassPlan &cp, int B, bool gmap);
@@ -106,10 +109,10 @@ struct NvtxRange {
     NvtxRange(const NvtxRange &) = delete;
     NvtxRange &operator=(const NvtxRange &) = delete;
 };
-// Packed classes store a successor as PED << 16 | parent slot << jbits | j with
-// jbits = bit length of n2 (j runs over 0..n2): a pair may be packed only if no PED reaches
-// 2^16 and its K fits the remaining 16 - jbits bits. The single-word kernels are always
-// packed; a single-word pair that is not packable is solved by the two-word kernels.
+// Single-word pairs go to the single-word kernels when no PED can reach 2^16 (the one-warp
+// kernel's entries hold 16-bit offsets, and the one-CTA kernel's padding columns score 2^29)
+// and K fits the 16 - jbits bits left beside a target vertex in a 16-bit code, jbits being the
+// bit length of n2; the others are solved by the two-word kernels.
 inline int jbits_of(int n2)
 {
     int b = 0;

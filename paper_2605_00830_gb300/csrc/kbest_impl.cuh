@@ -3,10 +3,11 @@
 // live in kbest_kernels.cu).
 //
 //   kbest_kernel          S1-S5 for every pair of a size class: persistent one-CTA teams pull
-//                         pairs from a device work queue; per level they build per-node
-//                         neighbour bitsets, score every successor with AND/XOR + popcount
-//                         against the staged vertex-cost row, select the best K exactly
-//                         (a PED histogram, a stable compaction and a counting placement),
+//                         pairs from a device work queue; per level they find the target
+//                         vertices still open to some node, build per-node neighbour bitsets,
+//                         score every open (node, column) with AND/XOR + popcount into one
+//                         byte and one histogram count, select the best K exactly (threshold
+//                         bucket, a stable compaction of the bytes, a counting placement),
 //                         write the kept children in key order and stage the next cost row;
 //                         finally they complete the leaves and take the argmin.
 //   kbest_cluster_kernel  the same with a team of 2-16 CTAs in a thread-block cluster, for
@@ -65,13 +66,8 @@ __device__ __forceinline__ uint64_t low_mask(int i, int w)
 template <int MW>
 struct TeamSharedT {
     int pair;
-    int cnt;
-    int mx;
-    int wmin[MW];  // least successor PED each warp scored at this level
-    int wn[MW];    // successors each warp scored at this level
-    int wlt[MW];
-    int weq[MW];
-    unsigned long long wbest[MW];
+    int wcode[MW];                  // best successor of each warp (variant B)
+    unsigned long long wbest[MW];   // best completion key of each warp
 };
 using TeamShared = TeamSharedT<kMaxWarps>;
 using TeamSharedCl = TeamSharedT<kMaxClusterWarps>;
@@ -123,8 +119,11 @@ struct Team {
 
 template <typename Word>
 struct Regions {
-    int32_t *hist, *alpha2, *crow, *sbase, *sel, *selped, *klist, *kped, *noff, *nbr, *cand;
+    int32_t *hist, *alpha2, *crow, *sbase, *sel, *selped, *klist, *kped, *noff, *nbr, *chist;
     int32_t *ped0, *ped1;
+    uint32_t *allm;
+    uint16_t *act;
+    uint8_t *score, *rec;
     Word *a2t, *l2t, *img0, *img1, *P, *PL, *imgl;
     uint8_t *map0, *map1;
 };
@@ -159,146 +158,464 @@ __device__ __forceinline__ unsigned same_value_lanes(unsigned valid, const unsig
     return m;
 }
 
-// PED of successor entry k: a packed 32-bit entry (PED << 16 | parent slot << jbits | j) or
-// an unpacked 64-bit one (PED << 32 | parent slot << kSelShift | j).
-__device__ __forceinline__ int entry_ped(const KParams &p, const int32_t *cand, int64_t k, bool pk)
+// One active column of a level for the single-word teams: adjacency word and label planes of
+// the target vertex, its cost-row entry, padded to 16 bytes so that one vector load or two
+// bring it. All lanes of a warp read the same record (a broadcast).
+template <typename Word, int NPL>
+struct __align__(16) ColRec {
+    Word a2;
+    Word l[NPL > 0 ? NPL : 1];
+    int32_t crow;
+};
+
+static_assert(sizeof(ColRec<uint32_t, 0>) == col_rec_bytes(true, 0), "record size");
+static_assert(sizeof(ColRec<uint32_t, 2>) == col_rec_bytes(true, 2), "record size");
+static_assert(sizeof(ColRec<uint32_t, kMaxB>) == col_rec_bytes(true, kMaxB), "record size");
+static_assert(sizeof(ColRec<uint64_t, 0>) == col_rec_bytes(false, 0), "record size");
+static_assert(sizeof(ColRec<uint64_t, 2>) == col_rec_bytes(false, 2), "record size");
+static_assert(sizeof(ColRec<uint64_t, kMaxB>) == col_rec_bytes(false, kMaxB), "record size");
+
+// Score bytes: one per (parent node, active column) of the nodes a CTA owns, row after row.
+// 0..126 is the successor's PED offset from the pass's anchor (0 also stands for one below an
+// anchor that is a guess), 127 stands for an offset past
+// the window and for a column that is no successor of the node (its vertex is used).
+constexpr int kScoreMax = 127;
+constexpr int kAnchorSlack = 48;   // of the 127 offsets, kept for a level that starts lower
+constexpr int kBuckets = kHistRow;   // histogram counters: offsets 0..126, [127] the successors
+
+// Everything a warp needs to score its nodes at one level.
+template <typename Word>
+struct LevelView {
+    const Word *imgw;       // Img rows: the CTA's staged copy (cluster) or the beam's
+    const int32_t *crow;    // S1 cost row
+    int ioff, cs0;          // first node of imgw's rows, of the CTA's node tables
+    int s_lo, s_hi;         // nodes of this warp
+    int nact;               // active columns of the level
+    int stride;             // bytes per row of score bytes (>= nact)
+    int64_t nimg;           // elements behind imgw
+};
+
+// PED of successor (node s, column j). Column j == n2 is the deletion v_i -> eps: its A2
+// column is empty, so the implied-edge terms count every substituted neighbour in P as a
+// deleted edge (with the dcnt deleted neighbours in sbase, all deg edges to v_0..v_{i-1}),
+// and the cost row holds c_vdel there.
+template <int W, typename Word>
+__device__ __forceinline__ int succ_ped(const KParams &p, const Regions<Word> &R,
+                                        const LevelView<Word> &V, int B, int s, int j)
 {
-    return pk ? (int)(FG_AT((const uint32_t *)cand, k, FG_N(uint32_t, p.lay.rsize[RG_CAND])) >> 16)
-              : (int)(FG_AT((const uint64_t *)cand, k, FG_N(uint64_t, p.lay.rsize[RG_CAND])) >> 32);
+    const int64_t im = (int64_t)(s - V.ioff) * W, Ps = (int64_t)(s - V.cs0) * W;
+    const bool fold_ie = p.cost.eins == p.cost.edel;
+    const int N2S = p.lay.n2s;
+    int x = 0, y = 0, z = 0;
+    for (int w = 0; w < W; ++w) {
+        const Word aw = FG_AT(R.a2t, w * N2S + j, FG_N(Word, p.lay.rsize[RG_A2T]));
+        const Word ai = aw & FG_AT(V.imgw, im + w, V.nimg);
+        const Word pw = FG_AT(R.P, Ps + w, FG_N(Word, p.lay.rsize[RG_P]));
+        if (fold_ie) {
+            x += popcw((Word)(ai ^ pw));
+        } else {
+            x += popcw((Word)(ai & ~pw));
+            y += popcw((Word)(pw & ~aw));
+        }
+        Word ld = (Word)0;
+        for (int b = 0; b < B; ++b)
+            ld |= FG_AT(R.PL, ((int64_t)b * p.lay.kloc + (s - V.cs0)) * W + w, FG_N(Word, p.lay.rsize[RG_PL])) ^
+                  FG_AT(R.l2t, (b * W + w) * N2S + j, FG_N(Word, p.lay.rsize[RG_L2T]));
+        z += popcw((Word)(aw & pw & ld));
+    }
+    return FG_AT(R.sbase, s - V.cs0, FG_N(int32_t, p.lay.rsize[RG_SBASE])) +
+           FG_AT(V.crow, j, N2S) + p.cost.eins * x + p.cost.edel * y + p.cost.esub * z;
 }
 
-// Stable compaction of the kept successors of this warp, in enumeration order: every
-// candidate with PED < T, and the first q with PED == T counted over the whole team.
-// keep_before / eq_before: kept / tied candidates of the warps before this one.
-template <typename Word>
-__device__ __forceinline__ int compact_kept(const KParams &p, const Regions<Word> &R, int base,
-                                           int n, int T, int q, int keep_before, int eq_before,
-                                           bool pk)
+// S3 over nodes [g0, g0 + ng) of this warp, lanes <-> active columns.
+//
+// Bound: the integer pipes. A column costs W popcounts of 64 bits (two 32-bit POPC each, 16
+// lanes per clock and SM), so a chunk of 32 columns takes at least 4 W clocks of an SM. Only
+// columns some node still has free are scored (1.02-1.3 times the free ones on dense and
+// large pairs, 2.1 times on a beam of 20,000). A score leaves one byte instead of the 8-byte
+// entry that was written once and read back twice, and its histogram count is taken here: a
+// shared increment costs 6 clocks of an SM per warp for any mix of buckets, what counting in
+// packed registers costs too, but on the memory pipe. 1,024 dense pairs of 50-200 vertices,
+// K = 256: 41.9 -> 19.6 ms; 64 pairs of 500-1,000 vertices, K = 1,024: 554 -> 327 ms; one
+// G(200, 0.4) pair, K = 5,000: 40.1 -> 29.3 ms.
+//
+// Every column's target
+// tables stay in registers while the warp walks its nodes, whose vectors are read as
+// broadcasts. With few active columns a warp scores several nodes per step. Each score leaves
+// one byte and one count in the warp's histogram row (a shared-memory increment, which the
+// hardware aggregates over lanes with the same bucket).
+// EXACT = 0: offset from `anchor`, offsets below it counting as 0. EXACT = 1 (selection
+// past the histogram window): sh >= 0 gives (PED - anchor) >> sh with PEDs below the anchor
+// left out; sh < 0 marks 0 = below the anchor, 1 = at the anchor, 127 = above.
+template <int W, typename Word, int BK, bool FOLD, bool EXACT>
+__device__ __forceinline__ void score_nodes(const KParams &p, const Regions<Word> &R,
+                                            const LevelView<Word> &V, int B, int n2, int nw,
+                                            int g0, int ng, int anchor, int sh, int32_t *hrow)
 {
+    constexpr int WB = 8 * (int)sizeof(Word);
+    constexpr int NPL = BK == 8 ? kMaxB : BK;
+    constexpr bool kRegLab = W * NPL <= 4;   // label planes of a column held in registers
     const int lane = threadIdx.x & 31;
-    const int keep0 = keep_before;
-
-    // four chunks of 32 per step: their loads and threshold ballots are independent, so only
-    // chunks holding a kept candidate pay for the ordered part
-    for (int kb = 0; kb < n; kb += 128) {
-        int v[4];
-        unsigned le[4];
+    const int N2S = p.lay.n2s, KM = p.lay.kloc, nact = V.nact;
+    const int c_eins = p.cost.eins, c_edel = p.cost.edel, c_esub = p.cost.esub;
+    // columns per node in a step: 32, or a power of two that covers the active ones
+    const int cs = nact > 16 ? 5 : nact > 8 ? 4 : nact > 4 ? 3 : nact > 2 ? 2 : nact > 1 ? 1 : 0;
+    const int step = 32 >> cs, sub = lane >> cs;
+    for (int a0 = 0; a0 < nact; a0 += 1 << cs) {
+        const int a = a0 + (lane & ((1 << cs) - 1));
+        const bool col = a < nact;
+        const int j = col ? (int)FG_AT(R.act, a, FG_N(uint16_t, p.lay.rsize[RG_ACT])) : n2;
+        const int jw = min(j >> 5, W * WB / 32 - 1);
+        const uint32_t jm = j < n2 ? 1u << (j & 31) : 0u;   // 0: the deletion is never used up
+        Word aw[W], lw[kRegLab && NPL > 0 ? W * NPL : 1];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int k = kb + 32 * u + lane;
-            v[u] = k < n ? entry_ped(p, R.cand, (int64_t)base + k, pk) : INT_MAX;
+        for (int w = 0; w < W; ++w)
+            aw[w] = FG_AT(R.a2t, w * N2S + j, FG_N(Word, p.lay.rsize[RG_A2T]));
+        if (kRegLab && NPL > 0) {
+#pragma unroll
+            for (int x = 0; x < W * NPL; ++x)
+                lw[x] = x < B * W ? FG_AT(R.l2t, x * N2S + j, FG_N(Word, p.lay.rsize[RG_L2T])) : (Word)0;
         }
+        const int cj = FG_AT(V.crow, j, N2S) - anchor;
+#pragma unroll 2
+        for (int t0 = 0; t0 < ng; t0 += step) {
+            const bool ok = col && t0 + sub < ng;
+            const int s = g0 + (t0 + sub < ng ? t0 + sub : 0);
+            const int64_t im = (int64_t)(s - V.ioff) * W, Ps = (int64_t)(s - V.cs0) * W;
+            int x = 0, y = 0, z = 0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) le[u] = __ballot_sync(0xffffffffu, v[u] <= T);
-        if ((le[0] | le[1] | le[2] | le[3]) == 0u) continue;
+            for (int w = 0; w < W; ++w) {
+                if (W > 4 && w >= nw) break;
+                const Word ai = aw[w] & FG_AT(V.imgw, im + w, V.nimg);
+                const Word pw = FG_AT(R.P, Ps + w, FG_N(Word, p.lay.rsize[RG_P]));
+                if (FOLD) {
+                    x += popcw((Word)(ai ^ pw));
+                } else {
+                    x += popcw((Word)(ai & ~pw));
+                    y += popcw((Word)(pw & ~aw[w]));
+                }
+                if (NPL > 0 && B > 0) {
+                    Word ld = (Word)0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (le[u] == 0u) continue;
-            const bool is_eq = (v[u] == T);
-            const unsigned eqb = __ballot_sync(0xffffffffu, is_eq);
-            const int eq_rank = eq_before + __popc(eqb & lanemask_lt());
-            const bool keep = (v[u] < T) || (is_eq && eq_rank < q);
-            const unsigned kbm = __ballot_sync(0xffffffffu, keep);
-            if (keep) {
-                const int pos = keep_before + __popc(kbm & lanemask_lt());
-                FG_AT(R.klist, pos, FG_N(int32_t, p.lay.rsize[RG_KLIST])) = base + kb + 32 * u + lane;
-                FG_AT(R.kped, pos, FG_N(int32_t, p.lay.rsize[RG_KPED])) = v[u];
+                    for (int b = 0; b < NPL; ++b)
+                        if (b < B)
+                            ld |= FG_AT(R.PL, ((int64_t)b * KM + (s - V.cs0)) * W + w, FG_N(Word, p.lay.rsize[RG_PL])) ^
+                                  (kRegLab ? lw[kRegLab ? b * W + w : 0]
+                                           : FG_AT(R.l2t, (b * W + w) * N2S + j, FG_N(Word, p.lay.rsize[RG_L2T])));
+                    z += popcw((Word)(aw[w] & pw & ld));
+                }
             }
-            keep_before += __popc(kbm);
-            eq_before += __popc(eqb);
+            int d = FG_AT(R.sbase, s - V.cs0, FG_N(int32_t, p.lay.rsize[RG_SBASE])) + cj + c_eins * x;
+            if (!FOLD) d += c_edel * y;
+            if (NPL > 0) d += c_esub * z;
+            const uint32_t uw = FG_AT((const uint32_t *)V.imgw, im * (int)(sizeof(Word) / 4) + jw,
+                                      V.nimg * (int)(sizeof(Word) / 4));
+            int v;
+            if (EXACT) {
+                if (sh >= 0) v = d < 0 ? kScoreMax : min(d >> sh, kScoreMax);
+                else v = d < 0 ? 0 : d == 0 ? 1 : kScoreMax;
+            } else {
+                v = max(0, min(d, kScoreMax));
+            }
+            if (uw & jm) v = kScoreMax;
+            if (ok) {
+                FG_AT(R.score, (int64_t)(s - V.cs0) * V.stride + a, FG_N(uint8_t, p.lay.rsize[RG_SCORE])) = (uint8_t)v;
+                if (v < kScoreMax) atomicAdd(&FG_AT(hrow, v, kBuckets), 1);
+            }
         }
     }
-    return keep_before - keep0;
 }
 
-// Exact selection used when the kept set reaches past the histogram window: the K-th
-// smallest PED is found by bisection over team-wide counts, the kept candidates are
-// compacted stably, and ranked by (PED, enumeration order); sel receives successor indices.
-template <typename MapT, typename Word, bool CL, typename TS>
-__device__ __noinline__ void select_exact(const KParams &p, int32_t *cand, int32_t *klist,
-                                          int32_t *kped, int32_t *sel, int32_t *selped, TS &S,
-                                          int L, int stride, int newL, int lo, bool pk)
+// S3 for single-word teams, lanes <-> parent nodes. With 10-40 target vertices a chunk of 32
+// columns is half empty (1.9-2.3 lane slots per successor measured on the workload's levels)
+// and every node's vectors are loaded per chunk; this way round it is 1.6, the column records
+// are broadcasts, and four scores make one store (4,096 served molecule pairs, a third of them
+// with K = 512 here: 3.51 -> 2.98 ms). A node's vectors stay in its lane's
+// registers and the warp walks the level's active columns four at a time (one store of four
+// score bytes). A group of at most 16 nodes is spread over the lanes, 2^qs lanes per node
+// taking every 2^qs-th quad. nd: the lane's node in the group (valid when `act`), base: its
+// base PED less the anchor. Rows are an odd number of quads long, so the lanes' stores fall
+// into different banks.
+template <typename Word, int BK, bool FOLD>
+__device__ __forceinline__ void score_quads(const KParams &p, const Regions<Word> &R,
+                                            const LevelView<Word> &V, int B, int row, bool act,
+                                            int r, int qs, Word im, Word P, const Word *PL,
+                                            int base, int32_t *hrow)
+{
+    constexpr int NPL = BK == 8 ? kMaxB : BK;
+    using Rec = ColRec<Word, NPL>;
+    const Rec *rec = (const Rec *)R.rec;
+    const Word *jm = (const Word *)((const uint8_t *)R.rec + p.lay.jm_off);
+    const int c_eins = p.cost.eins, c_edel = p.cost.edel, c_esub = p.cost.esub;
+    const int nq = V.stride >> 2;
+    for (int k = r; k < nq; k += 1 << qs) {
+        uint32_t v4 = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const Rec c = FG_AT(rec, 4 * k + u, FG_N(Rec, p.lay.jm_off));
+            const Word used = im & FG_AT(jm, 4 * k + u, FG_N(Word, p.lay.rsize[RG_REC] - p.lay.jm_off));
+            const Word ai = c.a2 & im;
+            int d = base + c.crow;
+            if (FOLD) d += c_eins * popcw((Word)(ai ^ P));
+            else d += c_eins * popcw((Word)(ai & ~P)) + c_edel * popcw((Word)(P & ~c.a2));
+            if (NPL > 0) {
+                Word ld = (Word)0;
+#pragma unroll
+                for (int b = 0; b < NPL; ++b)
+                    if (b < B) ld |= PL[b] ^ c.l[b];
+                d += c_esub * popcw((Word)(c.a2 & P & ld));
+            }
+            const int v = used ? kScoreMax : max(0, min(d, kScoreMax));
+            if (act && v < kScoreMax) atomicAdd(&FG_AT(hrow, v, kBuckets), 1);
+            v4 |= (uint32_t)v << (8 * u);
+        }
+        if (act) FG_AT((uint32_t *)R.score, (int64_t)row * nq + k, FG_N(uint32_t, p.lay.rsize[RG_SCORE])) = v4;
+    }
+}
+
+// Scores this warp's nodes again for the exact selection (the node vectors are in place).
+template <int W, typename Word, int BK>
+__device__ __noinline__ void score_exact(const KParams &p, const Regions<Word> &R,
+                                         const LevelView<Word> &V, int B, int n2, int nw,
+                                         int anchor, int sh, int32_t *hrow)
+{
+    const int lane = threadIdx.x & 31;
+    for (int b = lane; b < kBuckets; b += 32) FG_AT(hrow, b, kBuckets) = 0;
+    __syncwarp();
+    if (p.cost.eins == p.cost.edel)
+        score_nodes<W, Word, BK, true, true>(p, R, V, B, n2, nw, V.s_lo, V.s_hi - V.s_lo, anchor, sh, hrow);
+    else
+        score_nodes<W, Word, BK, false, true>(p, R, V, B, n2, nw, V.s_lo, V.s_hi - V.s_lo, anchor, sh, hrow);
+    __syncwarp();
+}
+
+// Turns the warps' histogram rows into exclusive prefixes over the team's warps (in
+// enumeration order) and leaves the bucket totals in the row after the CTA's last warp.
+// A cluster's CTAs exchange their totals through its global scratch.
+template <bool CL, typename Word>
+__device__ __forceinline__ void prefix_buckets(const KParams &p, const Regions<Word> &R,
+                                               const Team<CL> &tm)
+{
+    const int nwl = (int)blockDim.x >> 5;
+    const int64_t NH = FG_N(int32_t, p.lay.rsize[RG_HIST]);
+    __syncthreads();
+    if (CL) {
+        const int cr = (int)cluster_rank();
+        for (int b = threadIdx.x; b < kBuckets; b += blockDim.x) {
+            int t = 0;
+            for (int w = 0; w < nwl; ++w) t += FG_AT(R.hist, w * kBuckets + b, NH);
+            FG_AT(R.chist, cr * kBuckets + b, FG_N(int32_t, p.lay.rsize[RG_CHIST])) = t;
+        }
+        tm.sync();
+    }
+    for (int b = threadIdx.x; b < kBuckets; b += blockDim.x) {
+        int run = 0, all = 0;
+        if (CL) {
+            const int cr = (int)cluster_rank(), ncta = (int)cluster_size();
+            for (int c0 = 0; c0 < ncta; c0 += 4) {   // four loads in flight
+                int v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    v[u] = c0 + u < ncta ? FG_AT(R.chist, (c0 + u) * kBuckets + b, FG_N(int32_t, p.lay.rsize[RG_CHIST])) : 0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    all += v[u];
+                    run += c0 + u < cr ? v[u] : 0;
+                }
+            }
+        }
+        for (int w = 0; w < nwl; ++w) {
+            const int t = FG_AT(R.hist, w * kBuckets + b, NH);
+            FG_AT(R.hist, w * kBuckets + b, NH) = run;
+            run += t;
+        }
+        FG_AT(R.hist, nwl * kBuckets + b, NH) = CL ? all : run;
+    }
+    __syncthreads();
+}
+
+// The bucket where the cumulative count reaches `want` (kScoreMax when it lies past the
+// window), the successors below it, and the lowest bucket that holds any. Lane l holds
+// buckets 4l..4l+3.
+__device__ __forceinline__ void find_threshold(const KParams &p, const int32_t *htot, int want,
+                                               int &thr, int &below, int &first)
+{
+    const int lane = threadIdx.x & 31;
+    int c[4], sum = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        c[u] = 4 * lane + u < kScoreMax ? FG_AT(htot, 4 * lane + u, kBuckets) : 0;
+        sum += c[u];
+    }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    int run = incl - sum, mt = kScoreMax, mb = 0, mf = kScoreMax;
+#pragma unroll
+    for (int u = 3; u >= 0; --u)
+        if (c[u]) mf = 4 * lane + u;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        if (mt == kScoreMax && run < want && run + c[u] >= want) {
+            mt = 4 * lane + u;
+            mb = run;
+        }
+        run += c[u];
+    }
+    thr = (int)__reduce_min_sync(0xffffffffu, (unsigned)mt);
+    first = (int)__reduce_min_sync(0xffffffffu, (unsigned)mf);
+    below = __shfl_sync(0xffffffffu, mb, (thr >> 2) & 31);   // of the lane that holds thr
+}
+
+// Stable compaction of this warp's kept successors, in enumeration order (the order of its
+// score bytes): every byte below `thr`, and the first q bytes equal to it counted over the
+// whole team. 16 bytes per lane and step. klist receives (parent slot << kSelShift) | j and
+// kped the byte, from position `pos`; eq: tied successors of the warps before this one.
+template <typename Word>
+__device__ __forceinline__ int compact_kept(const KParams &p, const Regions<Word> &R,
+                                            const LevelView<Word> &V, int thr, int q, int pos,
+                                            int eq)
+{
+    const int lane = threadIdx.x & 31;
+    const int pos0 = pos;
+    const int64_t lo = (int64_t)(V.s_lo - V.cs0) * V.stride, hi = (int64_t)(V.s_hi - V.cs0) * V.stride;
+    const uint32_t t4 = (uint32_t)thr * 0x01010101u;
+    for (int64_t b0 = lo & ~(int64_t)15; b0 < hi; b0 += 512) {
+        const int64_t o = b0 + 16 * lane;
+        uint32_t le[4] = {0, 0, 0, 0}, eqm[4] = {0, 0, 0, 0}, v[4] = {0, 0, 0, 0};
+        if (o < hi) {
+            const uint4 x = FG_AT((const uint4 *)R.score, o >> 4, FG_N(uint4, p.lay.rsize[RG_SCORE]));
+            v[0] = x.x;
+            v[1] = x.y;
+            v[2] = x.z;
+            v[3] = x.w;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                // bytes are at most 127: bit 7 of a byte says byte <= thr, byte == thr
+                le[u] = ((t4 | 0x80808080u) - v[u]) & 0x80808080u;
+                eqm[u] = (0x80808080u - (v[u] ^ t4)) & 0x80808080u;
+            }
+            if (o < lo || o + 16 > hi) {   // bytes of the warps before and after this one
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    uint32_t m = 0;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int64_t at = o + 4 * u + k;
+                        if (at >= lo && at < hi) m |= 0x80u << (8 * k);
+                    }
+                    le[u] &= m;
+                    eqm[u] &= m;
+                }
+            }
+        }
+        const int nle = __popc(le[0]) + __popc(le[1]) + __popc(le[2]) + __popc(le[3]);
+        if (!__any_sync(0xffffffffu, nle > 0)) continue;
+        const int neq = __popc(eqm[0]) + __popc(eqm[1]) + __popc(eqm[2]) + __popc(eqm[3]);
+        int incl = (nle - neq) | (neq << 16);   // at most 512 each
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, s);
+            if (lane >= s) incl += y;
+        }
+        const int all = __shfl_sync(0xffffffffu, incl, 31);
+        if (nle > 0) {
+            int e = eq + (incl >> 16) - neq;                  // ties before this lane
+            int at = pos + (incl & 0xffff) - (nle - neq) + (min(e, q) - min(eq, q));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                uint32_t m = le[u];
+                while (m) {
+                    const int bit = __ffs((int)m) - 1;
+                    m &= m - 1u;
+                    const bool tie = (eqm[u] >> bit) & 1u;
+                    if (tie && e++ >= q) continue;
+                    const uint32_t idx = (uint32_t)(o + 4 * u + (bit >> 3));
+                    const uint32_t row = idx / (uint32_t)V.stride;
+                    const int j = (int)FG_AT(R.act, idx - row * (uint32_t)V.stride, FG_N(uint16_t, p.lay.rsize[RG_ACT]));
+                    FG_AT(R.klist, at, FG_N(int32_t, p.lay.rsize[RG_KLIST])) = ((V.cs0 + (int)row) << kSelShift) | j;
+                    FG_AT(R.kped, at, FG_N(int32_t, p.lay.rsize[RG_KPED])) = (int)((v[u] >> (bit & 24)) & 0xffu);
+                    ++at;
+                }
+            }
+        }
+        const int aeq = all >> 16;
+        pos += (all & 0xffff) + (min(eq + aeq, q) - min(eq, q));
+        eq += aeq;
+    }
+    return pos - pos0;
+}
+
+// Exact selection, used when the kept set reaches past the histogram window: the level is
+// scored again over coarser, then finer PED windows until the K-th PED is known exactly, the
+// kept candidates are compacted stably and ordered by (PED, enumeration order).
+// thr >= 0: offset of the K-th PED from `anchor`, with `below` successors below it.
+template <int W, typename Word, int BK, bool CL>
+__device__ __noinline__ void select_exact(const KParams &p, const Regions<Word> &R,
+                                          const LevelView<Word> &V, int B, int n2, int nw,
+                                          int newL, int anchor, int thr, int below)
 {
     const Team<CL> tm;
-    const int tid = tm.tid, lane = threadIdx.x & 31, warp = tm.warp;
-    const int T = tm.T, NW = tm.NW;
-    const int s_lo = (warp * L) / NW;
+    const int tid = tm.tid, T = tm.T, lane = threadIdx.x & 31;
+    const int nwl = (int)blockDim.x >> 5, lw = (int)threadIdx.x >> 5;
+    int32_t *hrow = R.hist + lw * kBuckets;
+    const int32_t *htot = R.hist + nwl * kBuckets;
 #define NKP FG_N(int32_t, p.lay.rsize[RG_KPED])
 #define NKL FG_N(int32_t, p.lay.rsize[RG_KLIST])
 #define NSE FG_N(int32_t, p.lay.rsize[RG_SEL])
 #define NSP FG_N(int32_t, p.lay.rsize[RG_SELPED])
-#define NSW ((int64_t)(sizeof(S.wn) / sizeof(S.wn[0])))
-    const int base = s_lo * stride, n = FG_AT(S.wn, warp, NSW);
-    Regions<Word> R;
-    R.cand = cand;
-    R.klist = klist;
-    R.kped = kped;
-
-    int mx = 0;
-    for (int k = lane; k < n; k += 32) mx = max(mx, entry_ped(p, cand, base + k, pk));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (tid == 0) S.mx = 0;
-    tm.sync();
-    if (lane == 0) atomicMax(&S.mx, mx);
-    tm.sync();
-    int hi = S.mx;
-    if (lo > hi) lo = hi;
-    // invariant: count(PED < lo) < newL <= count(PED <= hi)
-    while (lo < hi) {
-        const int mid = lo + (hi - lo) / 2;
-        int cnt = 0;
-        for (int k = lane; k < n; k += 32) cnt += (entry_ped(p, cand, base + k, pk) <= mid);
-        cnt = warp_sum(cnt);
-        tm.sync();
-        if (tid == 0) S.cnt = 0;
-        tm.sync();
-        if (lane == 0) atomicAdd(&S.cnt, cnt);
-        tm.sync();
-        if (S.cnt >= newL) hi = mid; else lo = mid + 1;
+    if (thr < 0) {
+        // windows of 127 buckets, each 64 times as wide as the one before, until one holds the
+        // K-th PED (PEDs are below 2^31, so a bucket width of 2^30 does); then 64 buckets of
+        // 1/64 the width inside the bucket found
+        int sh = 0, pre = 0, first;
+        bool down = false;
+        for (int pass = 0; pass < 12 && !(down && sh == 0); ++pass) {   // up to 30, then to 0
+            sh += down ? -6 : 6;
+            tm.sync();
+            score_exact<W, Word, BK>(p, R, V, B, n2, nw, anchor, sh, hrow);
+            prefix_buckets<CL>(p, R, tm);
+            find_threshold(p, htot, newL - pre, thr, below, first);
+            if (thr < kScoreMax) {
+                down = true;
+                pre += below;
+                anchor += thr << sh;
+            }
+        }
+        below = pre;
+    } else {
+        anchor += thr;
     }
-    const int thr = lo;
-    int nlt = 0, neq = 0;
-    for (int k = lane; k < n; k += 32) {
-        const int v = entry_ped(p, cand, base + k, pk);
-        nlt += (v < thr);
-        neq += (v == thr);
-    }
-    nlt = warp_sum(nlt);
-    neq = warp_sum(neq);
-    if (lane == 0) { FG_AT(S.wlt, warp, NSW) = nlt; FG_AT(S.weq, warp, NSW) = neq; }
+    const int q = newL - below;
     tm.sync();
-    // the warps' counts are read by all lanes at once (for a cluster team they live in
-    // global scratch, so a serial walk would pay one round trip per warp)
-    int lt_all = 0, keep_before = 0, eq_before = 0;
-    for (int w = lane; w < NW; w += 32) {
-        const int lt = FG_AT(S.wlt, w, NSW);
-        lt_all += lt;
-        if (w < warp) {
-            keep_before += lt;
-            eq_before += FG_AT(S.weq, w, NSW);
+    score_exact<W, Word, BK>(p, R, V, B, n2, nw, anchor, -1, hrow);
+    prefix_buckets<CL>(p, R, tm);
+    {
+        const int lt = FG_AT(hrow, 0, kBuckets), eq = FG_AT(hrow, 1, kBuckets);
+        const int kbeg = lt + min(q, eq);
+        const int kcnt = compact_kept<Word>(p, R, V, 1, q, kbeg, eq);
+        __syncwarp();
+        for (int x = kbeg + lane; x < kbeg + kcnt; x += 32) {
+            const int code = FG_AT(R.klist, x, NKL);
+            FG_AT(R.kped, x, NKP) = succ_ped<W, Word>(p, R, V, B, code >> kSelShift, code & ((1 << kSelShift) - 1));
         }
     }
-    lt_all = warp_sum(lt_all);
-    keep_before = warp_sum(keep_before);
-    eq_before = warp_sum(eq_before);
-    const int q = newL - lt_all;
-    keep_before += min(q, eq_before);
-    compact_kept<Word>(p, R, base, n, thr, q, keep_before, eq_before, pk);
     tm.sync();
-    // order by (PED, enumeration order); klist is in enumeration order and its entries are
+    // order by (PED, enumeration order); klist is in enumeration order and its codes are
     // increasing, so (kped, klist) is that key
     if (newL <= 2048) {
         for (int a = tid; a < newL; a += T) {
-            const int pa = FG_AT(kped, a, NKP);
+            const int pa = FG_AT(R.kped, a, NKP);
             int rank = 0;
             for (int b = 0; b < newL; ++b) {
-                const int pb = FG_AT(kped, b, NKP);
+                const int pb = FG_AT(R.kped, b, NKP);
                 rank += (pb < pa) || (pb == pa && b < a);
             }
-            // successor index; the caller turns it into (slot, j)
-            FG_AT(sel, rank, NSE) = FG_AT(klist, a, NKL);
-            FG_AT(selped, rank, NSP) = pa;
+            FG_AT(R.sel, rank, NSE) = FG_AT(R.klist, a, NKL);
+            FG_AT(R.selped, rank, NSP) = pa;
         }
         return;
     }
@@ -309,13 +626,13 @@ __device__ __noinline__ void select_exact(const KParams &p, int32_t *cand, int32
     while (N < newL) N <<= 1;
     auto cmpswap = [&](int i, int j) {
         if (j >= newL) return;
-        const int pi = FG_AT(kped, i, NKP), pj = FG_AT(kped, j, NKP);
-        const int li = FG_AT(klist, i, NKL), lj = FG_AT(klist, j, NKL);
+        const int pi = FG_AT(R.kped, i, NKP), pj = FG_AT(R.kped, j, NKP);
+        const int li = FG_AT(R.klist, i, NKL), lj = FG_AT(R.klist, j, NKL);
         if (pj < pi || (pj == pi && lj < li)) {
-            FG_AT(kped, i, NKP) = pj;
-            FG_AT(kped, j, NKP) = pi;
-            FG_AT(klist, i, NKL) = lj;
-            FG_AT(klist, j, NKL) = li;
+            FG_AT(R.kped, i, NKP) = pj;
+            FG_AT(R.kped, j, NKP) = pi;
+            FG_AT(R.klist, i, NKL) = lj;
+            FG_AT(R.klist, j, NKL) = li;
         }
     };
     for (int size = 2; size <= N; size <<= 1) {
@@ -335,14 +652,13 @@ __device__ __noinline__ void select_exact(const KParams &p, int32_t *cand, int32
         }
     }
     for (int a = tid; a < newL; a += T) {
-        FG_AT(sel, a, NSE) = FG_AT(klist, a, NKL);
-        FG_AT(selped, a, NSP) = FG_AT(kped, a, NKP);
+        FG_AT(R.sel, a, NSE) = FG_AT(R.klist, a, NKL);
+        FG_AT(R.selped, a, NSP) = FG_AT(R.kped, a, NKP);
     }
 #undef NKP
 #undef NKL
 #undef NSE
 #undef NSP
-#undef NSW
 }
 
 // BK: edge-label planes known at compile time: 0 (unlabelled), 2 (exactly two planes), or
@@ -364,25 +680,19 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
     const GraphMeta m1 = FG_AT(p.gmeta, g1, p.n_graphs), m2 = FG_AT(p.gmeta, g2, p.n_graphs);
     const int n1 = m1.n, n2 = m2.n, W1 = m1.W, W2 = m2.W;
     const int K = p.kpp ? FG_AT(p.kpp, pair, p.n_pairs) : p.K;
-    const int B = BK == 0 ? 0 : (BK == 2 ? 2 : p.lay.B);
+    const int Bc = BK == 0 ? 0 : (BK == 2 ? 2 : p.lay.B);   // planes of the class
     const int N2S = p.lay.n2s;
     const int KM = p.lay.kloc;   // node slots of the P / PL / sbase tables this CTA indexes
+    constexpr int W32 = W * (int)sizeof(Word) / 4;   // 32-bit words of a bitset
+    const int nwl = (int)blockDim.x >> 5;            // warps of this CTA
+    const int nw = min(W, max(1, (n2 + WB - 1) / WB));   // words this pair's bitsets use
+    int32_t *hrow = R.hist + (threadIdx.x >> 5) * kBuckets;   // this warp's histogram row
+    const int32_t *htot = R.hist + nwl * kBuckets;            // team totals (prefix_buckets)
     const int64_t mrow = p.lay.mrow;
-    const int stride = n2 + 1;   // successors of one node at most: n2 substitutions + deletion
     const MapT DEL = (MapT)~(MapT)0;
     const CostModel c = p.cost;
-    const int hwin = p.hwin;     // buckets 0..hwin-2 hold one PED each, hwin-1 the rest
+    const int hwin = p.hwin;     // PEDs a kept list may span without the exact selection
     const bool fold_ie = (c.eins == c.edel);
-    // Every successor is one entry of R.cand. Packed classes use 32 bits:
-    //   PED << 16 | parent slot << jbits | j,   jbits = bit length of n2 (j = 0..n2);
-    // the host packs a class only if no pair's PED can reach 2^16 and every K fits the slot
-    // field (K <= 2^(16 - jbits)); single-word classes are always packed. The others use
-    // 64 bits: PED << 32 | parent slot << kSelShift | j (the low half is the selection code).
-    const bool pk = CL ? false : (W == 1 ? true : p.lay.pk != 0);
-    const int jbits = 32 - __clz(n2);
-    const uint32_t jmask = (1u << jbits) - 1u;
-    uint32_t *ck = (uint32_t *)R.cand;
-    uint64_t *ck64 = (uint64_t *)R.cand;
     // lane-constant masks: lane b answers for histogram bucket b
     unsigned lanebit[5];
 #pragma unroll
@@ -394,6 +704,7 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
 
     // stage g2: transposed adjacency and label planes, vertex labels; g1 degrees (these
     // tables are per CTA)
+    bool lab = false;   // some edge of the pair has a label
     {
         const uint64_t *adj2 = p.adj + m2.adj_off;
         for (int idx = ltid; idx < W * n2; idx += LT) {
@@ -403,15 +714,16 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
                 (w64 < W2) ? (Word)(FG_AT(adj2, (int64_t)u * W2 + w64, p.adj_words - m2.adj_off) >> sh)
                            : (Word)0;
         }
-        for (int b = 0; b < B; ++b) {
+        for (int b = 0; b < Bc; ++b) {
             const uint64_t *pl2 = p.planes + m2.plane_off + (int64_t)b * n2 * W2;
             for (int idx = ltid; idx < W * n2; idx += LT) {
                 const int w = idx / n2, u = idx - w * n2;
                 const int w64 = (w * WB) >> 6, sh = (w * WB) & 63;
-                FG_AT(R.l2t, (b * W + w) * N2S + u, FG_N(Word, p.lay.rsize[RG_L2T])) =
-                    (w64 < W2) ? (Word)(FG_AT(pl2, (int64_t)u * W2 + w64,
-                                              p.plane_words - m2.plane_off - (int64_t)b * n2 * W2) >> sh)
-                               : (Word)0;
+                const Word l = (w64 < W2) ? (Word)(FG_AT(pl2, (int64_t)u * W2 + w64,
+                                                         p.plane_words - m2.plane_off - (int64_t)b * n2 * W2) >> sh)
+                                          : (Word)0;
+                FG_AT(R.l2t, (b * W + w) * N2S + u, FG_N(Word, p.lay.rsize[RG_L2T])) = l;
+                lab |= l != (Word)0;
             }
         }
         for (int u = ltid; u < n2; u += LT)
@@ -419,7 +731,7 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
         // column n2 of the target tables is the deletion v_i -> eps: no g2 neighbours, so the
         // substitution formula scores it with the deletion's edge costs (see succ_ped)
         for (int w = ltid; w < W; w += LT) FG_AT(R.a2t, w * N2S + n2, FG_N(Word, p.lay.rsize[RG_A2T])) = (Word)0;
-        for (int x = ltid; x < B * W; x += LT) FG_AT(R.l2t, x * N2S + n2, FG_N(Word, p.lay.rsize[RG_L2T])) = (Word)0;
+        for (int x = ltid; x < Bc * W; x += LT) FG_AT(R.l2t, x * N2S + n2, FG_N(Word, p.lay.rsize[RG_L2T])) = (Word)0;
         // S1 cost row of level 0 (the row of level i + 1 is written during level i)
         if (n1 > 0) {
             const int a10 = FG_AT(p.vlab, m1.lab_off, p.n_vlab);
@@ -436,6 +748,7 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
             FG_AT(R.noff, v + 1, FG_N(int32_t, p.lay.rsize[RG_NOFF])) = d;
         }
         if (ltid == 0) FG_AT(R.noff, 0, FG_N(int32_t, p.lay.rsize[RG_NOFF])) = 0;
+        for (int x = ltid; x < W32; x += LT) FG_AT(R.allm, x, FG_N(uint32_t, p.lay.rsize[RG_ALL])) = ~0u;
         // root node: empty lambda, R_V2 = V2, PED 0
         for (int w = tid; w < W; w += T) FG_AT(R.img0, w, FG_N(Word, p.lay.rsize[RG_IMG0])) = (Word)0;
         if (tid == 0) FG_AT(R.ped0, 0, FG_N(int32_t, p.lay.rsize[RG_PED0])) = 0;
@@ -468,435 +781,298 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
             while (bits) {
                 const int t = __ffsll((long long)bits) - 1;
                 bits &= bits - 1ull;
-                int lab = 0;
-                for (int b = 0; b < B; ++b)
-                    lab |= (int)((FG_AT(p.planes, pl + b * pstep + w, p.plane_words) >> t) & 1ull) << b;
-                FG_AT(R.nbr, o++, FG_N(int32_t, p.lay.rsize[RG_NBR])) = (w * 64 + t) | (lab << 16);
+                int el = 0;
+                for (int b = 0; b < Bc; ++b)
+                    el |= (int)((FG_AT(p.planes, pl + b * pstep + w, p.plane_words) >> t) & 1ull) << b;
+                lab |= el != 0;
+                FG_AT(R.nbr, o++, FG_N(int32_t, p.lay.rsize[RG_NBR])) = (w * 64 + t) | (el << 16);
             }
         }
     }
+    // a pair without edge labels in a labelled batch pays nothing for the planes
+    const int B = BK == 0 ? 0 : (__syncthreads_or(lab ? 1 : 0) ? Bc : 0);
     long long nevals = 0;
-    int L = 1;
+    int L = 1, rise = 0;
     // current / next beam buffers, swapped after every level
     uint8_t *mapc = R.map0, *mapn = R.map1;
     Word *imgc = R.img0, *imgn = R.img1;
     int32_t *pedc = R.ped0, *pedn = R.ped1;
     int32_t *crc = R.crow, *crn = R.crow + N2S;   // S1 cost rows of this level and the next
     // elements of the beam buffers (both buffers of a pair have the same size), the cost-row
-    // halves, the P / PL / sbase tables, the maps in MapT and 16-byte units, the entries
+    // halves, the P / PL / sbase tables, the maps in MapT and 16-byte units
 #define NIMG FG_N(Word, p.lay.rsize[RG_IMG0])
 #define NPED FG_N(int32_t, p.lay.rsize[RG_PED0])
-#define NSW ((int64_t)(sizeof(S.wn) / sizeof(S.wn[0])))   // warps the team scalars hold
+#define NSW ((int64_t)(sizeof(S.wbest) / sizeof(S.wbest[0])))   // warps the team scalars hold
 #define NP FG_N(Word, p.lay.rsize[RG_P])
 #define NMAPT FG_N(MapT, p.lay.rsize[RG_MAP0])
 #define NMAP16 FG_N(uint4, p.lay.rsize[RG_MAP0])
-#define NCK FG_N(uint32_t, p.lay.rsize[RG_CAND])
-#define NCK64 FG_N(uint64_t, p.lay.rsize[RG_CAND])
 #define NIMGW (CL ? FG_N(Word, p.lay.rsize[RG_IMGL]) : NIMG)
     tm.sync();
     PHASE_MARK(0);
 
     for (int i = 0; i < n1; ++i) {
         const int n0 = FG_AT(R.noff, i, FG_N(int32_t, p.lay.rsize[RG_NOFF])), deg = FG_AT(R.noff, i + 1, FG_N(int32_t, p.lay.rsize[RG_NOFF])) - n0;
-        const int s_lo = (warp * L) / NW, s_hi = ((warp + 1) * L) / NW;
-        const int base = s_lo * stride;              // this warp's successor storage
+        // 64-bit products: K can be 2^20 and a team 256 warps
+        const int s_lo = (int)((int64_t)warp * L / NW), s_hi = (int)((int64_t)(warp + 1) * L / NW);
         // node tables the warp prepares and evaluates are indexed from cs0: 0 for a one-CTA
-        // team; for a cluster, the first node of this CTA (its P, PL and sbase are CTA-local
-        // and its nodes' Img rows are staged into shared memory)
-        int cs0 = 0, ioff = 0;
+        // team; for a cluster, the first node of this CTA (its P, PL, sbase and score bytes
+        // are CTA-local and its nodes' Img rows are staged into shared memory)
+        int cs0 = 0, ioff = 0, cs1 = L;
         const Word *imgw = imgc;
         if (CL) {
-            const int nwl = (int)blockDim.x >> 5;
             const int r0 = (int)cluster_rank() * nwl;
-            cs0 = (r0 * L) / NW;
-            const int cs1 = ((r0 + nwl) * L) / NW;
-            for (int x = ltid; x < (cs1 - cs0) * W; x += LT)
-                FG_AT(R.imgl, x, FG_N(Word, p.lay.rsize[RG_IMGL])) = FG_AT(imgc, (int64_t)cs0 * W + x, NIMG);
-            __syncthreads();
+            cs0 = (int)((int64_t)r0 * L / NW);
+            cs1 = (int)((int64_t)(r0 + nwl) * L / NW);
             imgw = R.imgl;
             ioff = cs0;
         }
-        // ---- S1 + S2 per-node vectors, successor lists, S3 evaluation ----------------
-        int kw = 0;          // successors of this warp so far
-        int wmin = INT_MAX;  // least PED this warp scored
-        // PED of successor idx
-        auto ped_at = [&](int idx) -> int { return entry_ped(p, R.cand, idx, pk); };
-        // S3: PED of successor (node sc, column j). Column j == n2 is the deletion
-        // v_i -> eps: its A2 column is empty, so the implied-edge terms count every
-        // substituted neighbour in P as a deleted edge (with the dcnt deleted neighbours in
-        // sbase, all deg edges to v_0..v_{i-1}), and the cost row holds c_vdel there.
-        // successors scored during the id sweep (one-CTA teams, two to four words), else in
-        // a chunked pass
-        constexpr bool kFuseEval = !CL && W > 1 && W <= 4;
-        auto succ_ped = [&](int sc, int j) -> int {
-            const int64_t im = (int64_t)(sc - ioff) * W;   // the parent's Img row
-            const int64_t Ps = (int64_t)(sc - cs0) * W;    // and its row of R.P
-            int x = 0, y = 0, z = 0;
+        // target vertices that every node of this CTA uses: the beam's nodes share most of
+        // their ancestors, so the columns left are little more than a node's own successors.
+        // A thread reads one 32-bit word index of every row it visits (W32 divides the warp).
+        {
+            uint32_t am = ~0u;
+            const int64_t n32 = (int64_t)(cs1 - cs0) * W32, b32 = (int64_t)cs0 * W32;
+            for (int64_t x = ltid; x < n32; x += LT) {
+                const uint32_t v = FG_AT((const uint32_t *)imgc, b32 + x, NIMG * (int)(sizeof(Word) / 4));
+                if (CL) FG_AT((uint32_t *)R.imgl, x, NIMGW * (int)(sizeof(Word) / 4)) = v;
+                am &= v;
+            }
 #pragma unroll
-            for (int w = 0; w < W; ++w) {
-                const Word aw = FG_AT(R.a2t, w * N2S + j, FG_N(Word, p.lay.rsize[RG_A2T]));
-                const Word ai = aw & FG_AT(imgw, im + w, NIMGW);
-                const Word pw = FG_AT(R.P, Ps + w, NP);
-                if (fold_ie) {
-                    x += popcw((Word)(ai ^ pw));
-                } else {
-                    x += popcw((Word)(ai & ~pw));
-                    y += popcw((Word)(pw & ~aw));
-                }
-                if (B > 0) {
-                    Word ld = (Word)0;
-                    for (int b = 0; b < B; ++b)
-                        ld |= FG_AT(R.PL, ((int64_t)b * KM + (sc - cs0)) * W + w, FG_N(Word, p.lay.rsize[RG_PL])) ^
-                              FG_AT(R.l2t, (b * W + w) * N2S + j, FG_N(Word, p.lay.rsize[RG_L2T]));
-                    z += popcw((Word)(aw & pw & ld));
+            for (int o = 16; o >= W32; o >>= 1) am &= __shfl_xor_sync(0xffffffffu, am, o);
+            if (lane < W32) atomicAnd(&FG_AT(R.allm, lane, FG_N(uint32_t, p.lay.rsize[RG_ALL])), am);
+        }
+        __syncthreads();
+        // active columns, increasing: the vertices not used by all, and the deletion n2
+        int nact = n2 + 1, stride;
+        {
+            using Rec = ColRec<Word, (BK == 8 ? kMaxB : BK)>;
+            constexpr int NPL = BK == 8 ? kMaxB : BK;
+            Word *jm = (Word *)((uint8_t *)R.rec + p.lay.jm_off);   // one-hot vertex bits
+#define NJM FG_N(Word, p.lay.rsize[RG_REC] - p.lay.jm_off)
+            for (int w = 0; w < W32; ++w) nact -= __popc(FG_AT(R.allm, w, FG_N(uint32_t, p.lay.rsize[RG_ALL])));
+            for (int j = ltid; j <= n2; j += LT) {
+                int pos = j;
+                bool fr = true;
+                if (cs1 > cs0) {
+                    for (int w = 0; w < W32; ++w) {
+                        const uint32_t m = FG_AT(R.allm, w, FG_N(uint32_t, p.lay.rsize[RG_ALL]));
+                        if (w < (j >> 5)) pos -= __popc(m);
+                        if (w == (j >> 5)) {
+                            pos -= __popc(m & ((1u << (j & 31)) - 1u));
+                            fr = !((m >> (j & 31)) & 1u);
+                        }
+                    }
+                    if (fr) {
+                        FG_AT(R.act, pos, FG_N(uint16_t, p.lay.rsize[RG_ACT])) = (uint16_t)j;
+                        if (W == 1) {
+                            Rec c;
+                            c.a2 = FG_AT(R.a2t, j, FG_N(Word, p.lay.rsize[RG_A2T]));
+#pragma unroll
+                            for (int b = 0; b < NPL; ++b)
+                                c.l[b] = b < B ? FG_AT(R.l2t, b * N2S + j, FG_N(Word, p.lay.rsize[RG_L2T])) : (Word)0;
+                            c.crow = FG_AT(crc, j, N2S);
+                            FG_AT((Rec *)R.rec, pos, FG_N(Rec, p.lay.jm_off)) = c;
+                            FG_AT(jm, pos, NJM) = j < n2 ? (Word)1 << (j % WB) : (Word)0;
+                        }
+                    }
                 }
             }
-            return FG_AT(R.sbase, sc - cs0, FG_N(int32_t, p.lay.rsize[RG_SBASE])) + FG_AT(crc, j, N2S) +
-                   c.eins * x + c.edel * y + c.esub * z;
-        };
+            stride = nact;
+            // single-word rows: whole quads of columns, an odd number of them; the columns
+            // past the active ones score past every bucket
+            if (W == 1) {
+                stride = ((nact + 3) / 4 | 1) * 4;
+                for (int a = nact + ltid; cs1 > cs0 && a < stride; a += LT) {
+                    Rec c = {};
+                    c.crow = 1 << 29;
+                    FG_AT((Rec *)R.rec, a, FG_N(Rec, p.lay.jm_off)) = c;
+                    FG_AT(jm, a, NJM) = (Word)0;
+                }
+            }
+        }
+#undef NJM
+        LevelView<Word> V;
+        V.imgw = imgw;
+        V.crow = crc;
+        V.ioff = ioff;
+        V.cs0 = cs0;
+        V.s_lo = s_lo;
+        V.s_hi = s_hi;
+        V.nact = nact;
+        V.stride = stride;
+        V.nimg = NIMGW;
+        // anchor of the level's PED offsets. No child's PED is below the best parent's, but in
+        // dense graphs all lie far above it, at a distance that changes little from one level
+        // to the next: the window starts kAnchorSlack below where the last level's began. If
+        // that is too high, bucket 0 is not empty and the exact selection takes over.
+        const int A0 = FG_AT(pedc, 0, NPED);
+        const int A = A0 + max(0, rise - kAnchorSlack);
+        const bool last_b = p.variant == 1 && i == n1 - 1;
+        for (int b = lane; b < kBuckets; b += 32) FG_AT(hrow, b, kBuckets) = 0;
+        __syncthreads();
+        PHASE_MARK(7);
+        // ---- S1 + S2 per-node vectors, S3 scores and their histogram -------------------
+        int kw = 0;          // successors of this lane's nodes so far
         for (int g0 = s_lo; g0 < s_hi; g0 += 32) {
             const int ng = min(32, s_hi - g0);
             const int s = g0 + lane;
-            const bool act = lane < ng;
-            int cnt = 0;
-            if (act) {
+            constexpr int NPL = BK == 8 ? kMaxB : (BK == 2 ? 2 : 1);
+            Word pr = (Word)0, plr[NPL], imr = (Word)0;   // single-word node vectors
+            int nbase = 0;
+#pragma unroll
+            for (int b = 0; b < NPL; ++b) plr[b] = (Word)0;
+            if (lane < ng) {
                 // S2: P = images of the substituted g1 neighbours of v_i (their edge labels in
                 // bit-planes PL at the image positions); dcnt = deleted neighbours
                 const int64_t Ps = (int64_t)(s - cs0) * W;   // this node's row of R.P
                 const int64_t ms = (int64_t)s * (mrow / (int64_t)sizeof(MapT));   // its map row
                 int dcnt = 0;
-                if (W == 1) {
-                    constexpr int NPL = BK == 8 ? kMaxB : (BK == 2 ? 2 : 1);
-                    Word pr = (Word)0, plr[NPL];
+                if (W > 1) {
 #pragma unroll
-                    for (int b = 0; b < NPL; ++b) plr[b] = (Word)0;
-                    // four neighbours per step: list and map loads first, then the bits
-                    for (int t0 = 0; t0 < deg; t0 += 4) {
-                        int e[4];
-                        MapT phi[4];
+                    for (int w = 0; w < W; ++w) FG_AT(R.P, Ps + w, NP) = (Word)0;
+                    for (int b = 0; b < B; ++b)
+                        for (int w = 0; w < W; ++w) FG_AT(R.PL, ((int64_t)b * KM + (s - cs0)) * W + w, FG_N(Word, p.lay.rsize[RG_PL])) = (Word)0;
+                }
+                // several neighbours per step: list and map loads first, then the bits
+                constexpr int NU = W > 1 ? 8 : 4;
+                for (int t0 = 0; t0 < deg; t0 += NU) {
+                    int e[NU];
+                    MapT phi[NU];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) e[u] = t0 + u < deg ? FG_AT(R.nbr, n0 + t0 + u, FG_N(int32_t, p.lay.rsize[RG_NBR])) : -1;
+                    for (int u = 0; u < NU; ++u) e[u] = t0 + u < deg ? FG_AT(R.nbr, n0 + t0 + u, FG_N(int32_t, p.lay.rsize[RG_NBR])) : -1;
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            phi[u] = e[u] >= 0 ? FG_AT((const MapT *)mapc, ms + (e[u] & 0xffff), NMAPT) : DEL;
+                    for (int u = 0; u < NU; ++u)
+                        phi[u] = e[u] >= 0 ? FG_AT((const MapT *)mapc, ms + (e[u] & 0xffff), NMAPT) : DEL;
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const bool sub = phi[u] != DEL;
-                            dcnt += (e[u] >= 0 && !sub) ? 1 : 0;
+                    for (int u = 0; u < NU; ++u) {
+                        const bool sub = phi[u] != DEL;
+                        dcnt += (e[u] >= 0 && !sub) ? 1 : 0;
+                        if (W == 1) {
                             const Word pb = sub ? (Word)1 << ((int)phi[u] % WB) : (Word)0;
                             pr |= pb;
 #pragma unroll
                             for (int b = 0; b < NPL; ++b)
                                 if (b < B && ((e[u] >> (16 + b)) & 1)) plr[b] |= pb;
+                        } else if (sub) {
+                            const int pw = (int)phi[u] / WB;
+                            const Word pb = (Word)1 << ((int)phi[u] % WB);
+                            FG_AT(R.P, Ps + pw, NP) |= pb;
+                            for (int b = 0; b < B; ++b)
+                                if ((e[u] >> (16 + b)) & 1) FG_AT(R.PL, ((int64_t)b * KM + (s - cs0)) * W + pw, FG_N(Word, p.lay.rsize[RG_PL])) |= pb;
                         }
                     }
+                }
+                if (W == 1) {
                     FG_AT(R.P, Ps, NP) = pr;
 #pragma unroll
                     for (int b = 0; b < NPL; ++b)
                         if (b < B) FG_AT(R.PL, (int64_t)b * KM + (s - cs0), FG_N(Word, p.lay.rsize[RG_PL])) = plr[b];
-                } else {
-#pragma unroll
-                    for (int w = 0; w < W; ++w) FG_AT(R.P, Ps + w, NP) = (Word)0;
-                    for (int b = 0; b < B; ++b)
-                        for (int w = 0; w < W; ++w) FG_AT(R.PL, ((int64_t)b * KM + (s - cs0)) * W + w, FG_N(Word, p.lay.rsize[RG_PL])) = (Word)0;
-                    for (int t = 0; t < deg; ++t) {
-                        const int e = FG_AT(R.nbr, n0 + t, FG_N(int32_t, p.lay.rsize[RG_NBR]));
-                        const MapT phi = FG_AT((const MapT *)mapc, ms + (e & 0xffff), NMAPT);
-                        if (phi == DEL) { ++dcnt; continue; }
-                        const int pw = (int)phi / WB;
-                        const Word pb = (Word)1 << ((int)phi % WB);
-                        FG_AT(R.P, Ps + pw, NP) |= pb;
-                        for (int b = 0; b < B; ++b)
-                            if ((e >> (16 + b)) & 1) FG_AT(R.PL, ((int64_t)b * KM + (s - cs0)) * W + pw, FG_N(Word, p.lay.rsize[RG_PL])) |= pb;
-                    }
                 }
-                FG_AT(R.sbase, s - cs0, FG_N(int32_t, p.lay.rsize[RG_SBASE])) =
-                    FG_AT(pedc, s, NPED) + c.edel * dcnt;
+                nbase = FG_AT(pedc, s, NPED) + c.edel * dcnt;
+                FG_AT(R.sbase, s - cs0, FG_N(int32_t, p.lay.rsize[RG_SBASE])) = nbase;
                 const int64_t im = (int64_t)(s - ioff) * W;   // this node's Img row in imgw
                 int used = 0;
 #pragma unroll
                 for (int w = 0; w < W; ++w) used += popcw(FG_AT(imgw, im + w, NIMGW));
-                cnt = n2 - used + 1;   // free g2 vertices (R_V2) and the deletion
+                kw += n2 - used + 1;   // free g2 vertices (R_V2) and the deletion
+                if (W == 1) imr = FG_AT(imgw, im, NIMGW);
             }
-            int incl = cnt;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += v;
-            }
-            const int excl = incl - cnt;
-            const int gtot = __shfl_sync(0xffffffffu, incl, 31);
-            // successor ids in enumeration order: for each node the free g2 vertices in
-            // increasing order, then n2 for v_i -> eps. Single-word bitsets: each lane walks
-            // its own node's bits; wider ones: the warp sweeps each node's vertices 32 at a
-            // time and compacts the free ones with a ballot.
-            if (W == 1 && !CL) {
-                if (act) {
-                    int idx = base + kw + excl;
-                    Word x = ~FG_AT(imgw, (int64_t)(s - ioff) * W, NIMGW);
-                    if (n2 < WB) x &= n2 > 0 ? (((Word)1 << n2) - (Word)1) : (Word)0;
-                    while (x) {
-                        const int t = (WB == 64) ? __ffsll((long long)x) - 1 : __ffs((int)x) - 1;
-                        x &= x - (Word)1;
-                        FG_AT(ck, idx, NCK) = ((uint32_t)s << jbits) | (uint32_t)t;
-                        ++idx;
-                    }
-                    FG_AT(ck, idx, NCK) = ((uint32_t)s << jbits) | (uint32_t)n2;
-                }
-            } else {
-                // one-CTA teams with two to four words: the sweep scores each free vertex
-                // where it finds it and writes the whole entry (PED and id), so the entries
-                // are not read back for the evaluation. Otherwise it writes ids, scored by the
-                // chunked pass below, where every lane scores a free vertex: that pays off
-                // once an evaluation costs eight words, and for cluster teams, whose pairs
-                // (wide beams) can have fewer target vertices than a warp has lanes
-                __syncwarp();   // the group's node vectors (P, PL, base) are in place
-                for (int t = 0; t < ng; ++t) {
-                    const int st_ = g0 + t;
-                    const int64_t im = (int64_t)(st_ - ioff) * W;   // the node's Img row
-                    const int o0 = base + kw + __shfl_sync(0xffffffffu, excl, t);
-                    int pos = 0;
-                    for (int j0 = 0; j0 < n2; j0 += 32) {
-                        const int j = j0 + lane;
-                        const bool fr = j < n2 && !((FG_AT(imgw, im + j / WB, NIMGW) >> (j % WB)) & (Word)1);
-                        const unsigned bal = __ballot_sync(0xffffffffu, fr);
-                        if (fr) {
-                            const int idx = o0 + pos + __popc(bal & lanemask_lt());
-                            const int d = kFuseEval ? succ_ped(st_, j) : 0;
-                            if (kFuseEval) wmin = d < wmin ? d : wmin;
-                            if (pk) FG_AT(ck, idx, NCK) = ((uint32_t)d << 16) | ((uint32_t)st_ << jbits) | (uint32_t)j;
-                            else FG_AT(ck64, idx, NCK64) = ((uint64_t)(uint32_t)d << 32) | ((uint64_t)st_ << kSelShift) | (uint64_t)j;
-                        }
-                        pos += __popc(bal);
-                    }
-                    if (lane == 0) {
-                        const int d = kFuseEval ? succ_ped(st_, n2) : 0;
-                        if (kFuseEval) wmin = d < wmin ? d : wmin;
-                        if (pk) FG_AT(ck, o0 + pos, NCK) = ((uint32_t)d << 16) | ((uint32_t)st_ << jbits) | (uint32_t)n2;
-                        else FG_AT(ck64, o0 + pos, NCK64) = ((uint64_t)(uint32_t)d << 32) | ((uint64_t)st_ << kSelShift) | (uint64_t)n2;
-                    }
-                }
-            }
-            __syncwarp();
+            __syncwarp();   // the group's node vectors (P, PL, base) are in place
             PHASE_MARK(5);
+            if (W == 1 && !last_b) {
+                const int qs = ng > 16 ? 0 : ng > 8 ? 1 : ng > 4 ? 2 : ng > 2 ? 3 : ng > 1 ? 4 : 5;
+                const int nd = lane >> qs;   // this lane's node of the group
+                if (qs) {
+                    pr = __shfl_sync(0xffffffffu, pr, nd);
+                    imr = __shfl_sync(0xffffffffu, imr, nd);
+                    nbase = __shfl_sync(0xffffffffu, nbase, nd);
+#pragma unroll
+                    for (int b = 0; b < NPL; ++b) plr[b] = __shfl_sync(0xffffffffu, plr[b], nd);
+                }
+                const int r = lane & ((1 << qs) - 1);
+                if (fold_ie) score_quads<Word, BK, true>(p, R, V, B, g0 + nd - cs0, nd < ng, r, qs, imr, pr, plr, nbase - A, hrow);
+                else score_quads<Word, BK, false>(p, R, V, B, g0 + nd - cs0, nd < ng, r, qs, imr, pr, plr, nbase - A, hrow);
+                PHASE_MARK(1);
+            } else if (!last_b) {
+                if (fold_ie) score_nodes<W, Word, BK, true, false>(p, R, V, B, n2, nw, g0, ng, A, 0, hrow);
+                else score_nodes<W, Word, BK, false, false>(p, R, V, B, n2, nw, g0, ng, A, 0, hrow);
+                PHASE_MARK(1);
+            }
+        }
+        kw = warp_sum(kw);
+        if (lane == 0) FG_AT(hrow, kScoreMax, kBuckets) = kw;
+        if (ltid < W32) FG_AT(R.allm, ltid, FG_N(uint32_t, p.lay.rsize[RG_ALL])) = ~0u;   // for the next level
+        prefix_buckets<CL>(p, R, tm);
+        const int total = FG_AT(htot, kScoreMax, kBuckets);   // successors of the level
+        PHASE_MARK(2);
 
-            // U chunks of 32 successors per step, their id loads and PEDs independent
-            constexpr int U = 2;
-            for (int kb = 0; !kFuseEval && kb < gtot; kb += 32 * U) {
-                int scu[U], ju[U];
-                uint32_t idu[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int k = kb + 32 * u + lane;
-                    const int idx = base + kw + k;
-                    if (pk) {
-                        idu[u] = k < gtot ? FG_AT(ck, idx, NCK) : (((uint32_t)g0 << jbits) | (uint32_t)n2);
-                        scu[u] = (int)(idu[u] >> jbits);
-                        ju[u] = (int)(idu[u] & jmask);
-                    } else {
-                        idu[u] = k < gtot ? (uint32_t)FG_AT(ck64, idx, NCK64)
-                                          : (((uint32_t)g0 << kSelShift) | (uint32_t)n2);
-                        scu[u] = (int)(idu[u] >> kSelShift);
-                        ju[u] = (int)(idu[u] & ((1u << kSelShift) - 1u));
-                    }
-                }
-                int pu[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) pu[u] = succ_ped(scu[u], ju[u]);
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int k = kb + 32 * u + lane;
-                    if (k < gtot) {
-                        if (pk) FG_AT(ck, base + kw + k, NCK) = ((uint32_t)pu[u] << 16) | idu[u];
-                        else FG_AT(ck64, base + kw + k, NCK64) = ((uint64_t)(uint32_t)pu[u] << 32) | idu[u];
-                        wmin = pu[u] < wmin ? pu[u] : wmin;
-                    }
-                }
-            }
-            kw += gtot;
-            __syncwarp();
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) wmin = min(wmin, __shfl_xor_sync(0xffffffffu, wmin, o));
-        if (lane == 0) {
-            FG_AT(S.wmin, warp, NSW) = wmin;
-            FG_AT(S.wn, warp, NSW) = kw;
-        }
-        tm.sync();
-        // S4 histogram of PED - pa over this warp's successors, pa = least PED of the level
-        // (the last bucket collects every PED past the window). Ballot counting: lane b keeps
-        // the count of bucket b; lanes past the end count in the last bucket, which only
-        // bounds the threshold search from above (the level total comes from the counts kw).
-        int pa = INT_MAX;
-        for (int w = lane; w < NW; w += 32) pa = min(pa, FG_AT(S.wmin, w, NSW));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) pa = min(pa, __shfl_xor_sync(0xffffffffu, pa, o));
-        {
-            int hreg = 0;
-            if (kw >= 1024 && kw <= 65000) {
-                // many candidates: each lane counts its own in 4-bit fields (two 64-bit words
-                // for 32 buckets), widened every 12 chunks into 16-bit fields, then a five-
-                // round shuffle reduce-scatter leaves bucket b's warp total in lane b (16-bit
-                // fields hold it: the warp has at most 65,000 candidates plus padding)
-                unsigned long long c0 = 0ull, c1 = 0ull, acc[8];
-#pragma unroll
-                for (int m = 0; m < 8; ++m) acc[m] = 0ull;
-                int pending = 0;
-                for (int kb = 0; kb < kw; kb += 128) {
-                    int d4[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int k = kb + 32 * u + lane;
-                        d4[u] = k < kw ? min(ped_at(base + k) - pa, hwin - 1) : hwin - 1;
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const unsigned long long inc = 1ull << (4 * (d4[u] & 15));
-                        if (d4[u] < 16) c0 += inc; else c1 += inc;
-                    }
-                    pending += 4;
-                    if (pending >= 12 || kb + 128 >= kw) {
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) {
-                            acc[m] += (c0 >> (4 * m)) & 0x000F000F000F000Full;
-                            acc[4 + m] += (c1 >> (4 * m)) & 0x000F000F000F000Full;
-                        }
-                        c0 = c1 = 0ull;
-                        pending = 0;
-                    }
-                }
-                const bool b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1;
-                const bool b1 = (lane >> 1) & 1, b0 = lane & 1;
-                unsigned q[4];
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    const unsigned long long send = b4 ? acc[m] : acc[4 + m];
-                    const unsigned long long keep = b4 ? acc[4 + m] : acc[m];
-                    const unsigned long long r = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-                    const unsigned lo = (unsigned)r, hi = (unsigned)(r >> 32);
-                    q[m] = (b3 ? hi : lo) + __shfl_xor_sync(0xffffffffu, b3 ? lo : hi, 8);
-                }
-                unsigned t[4];
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    const unsigned lo = q[m] & 0xffffu, hi = q[m] >> 16;
-                    t[m] = (b2 ? hi : lo) + __shfl_xor_sync(0xffffffffu, b2 ? lo : hi, 4);
-                }
-                unsigned u2[2];
-#pragma unroll
-                for (int m = 0; m < 2; ++m)
-                    u2[m] = (b1 ? t[2 + m] : t[m]) + __shfl_xor_sync(0xffffffffu, b1 ? t[m] : t[2 + m], 2);
-                hreg = (int)((b0 ? u2[1] : u2[0]) + __shfl_xor_sync(0xffffffffu, b0 ? u2[0] : u2[1], 1));
-            } else
-            // few candidates: five bit ballots per chunk, lane b counts the lanes whose
-            // bucket is b
-            for (int kb = 0; kb < kw; kb += 128) {
-                int d4[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int k = kb + 32 * u + lane;
-                    d4[u] = k < kw ? min(ped_at(base + k) - pa, hwin - 1) : hwin - 1;
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (kb + 32 * u >= kw) break;
-                    unsigned m = 0xffffffffu;
-#pragma unroll
-                    for (int b = 0; b < 5; ++b)
-                        m &= ~(__ballot_sync(0xffffffffu, (d4[u] >> b) & 1) ^ lanebit[b]);
-                    hreg += __popc(m);
-                }
-            }
-            FG_AT(R.hist, lane * NW + warp, FG_N(int32_t, p.lay.rsize[RG_HIST])) = hreg;
-        }
-        tm.sync();
-        PHASE_MARK(1);
-        // (parent slot << kSelShift) | j of successor idx
-        auto decode = [&](int idx) -> int {
-            if (pk) {
-                const uint32_t id = FG_AT(ck, idx, NCK) & 0xffffu;
-                return (int)((id >> jbits) << kSelShift) | (int)(id & jmask);
-            } else {
-                return (int)(uint32_t)FG_AT(ck64, idx, NCK64);
-            }
-        };
-
-        if (p.variant == 1 && i == n1 - 1) {
+        if (last_b) {
             // variant B: every successor of the last level is completed (insertions of the
             // free g2 vertices and their edges) and the least (total, PED, enumeration order)
-            // wins. Per node: nimg = |Img|, e2 = g2 edges inside Img (kept in klist / kped,
-            // which the selection does not use at this level).
-            for (int t = lane; t < s_hi - s_lo; t += 32) {
-                const int sl = s_lo + t;
-                const int64_t im = (int64_t)sl * W;   // the node's Img row
+            // wins. Lanes <-> active columns; per node: nimg = |Img|, e2 = g2 edges inside Img.
+            unsigned long long key = ~0ull;   // total << 32 | PED
+            int code = INT_MAX;               // parent slot << kSelShift | j
+            for (int s = s_lo; s < s_hi; ++s) {
+                const int64_t im = (int64_t)(s - ioff) * W;   // the node's Img row
                 int nimg = 0, acc = 0;
+                for (int u = lane; u < n2; u += 32) {
+                    if ((FG_AT(imgw, im + u / WB, NIMGW) >> (u % WB)) & (Word)1) {
+                        ++nimg;
 #pragma unroll
-                for (int w = 0; w < W; ++w) {
-                    Word x = FG_AT(imgc, im + w, NIMG);
-                    nimg += popcw(x);
-                    while (x) {
-                        const int bt = (WB == 64) ? __ffsll((long long)x) - 1 : __ffs((int)x) - 1;
-                        x &= x - (Word)1;
-                        const int u = w * WB + bt;
-#pragma unroll
-                        for (int w2 = 0; w2 < W; ++w2)
-                            acc += popcw((Word)(FG_AT(R.a2t, w2 * N2S + u, FG_N(Word, p.lay.rsize[RG_A2T])) &
-                                                FG_AT(imgc, im + w2, NIMG)));
+                        for (int w = 0; w < W; ++w)
+                            acc += popcw((Word)(FG_AT(R.a2t, w * N2S + u, FG_N(Word, p.lay.rsize[RG_A2T])) &
+                                                FG_AT(imgw, im + w, NIMGW)));
                     }
                 }
-                FG_AT(R.kped, sl, FG_N(int32_t, p.lay.rsize[RG_KPED])) = nimg;
-                FG_AT(R.klist, sl, FG_N(int32_t, p.lay.rsize[RG_KLIST])) = acc / 2;
-            }
-            __syncwarp();
-            auto leaf_total = [&](int k) -> long long {
-                const int idx = base + k;
-                const int v = decode(idx);
-                const int sc = v >> kSelShift, j = v & ((1 << kSelShift) - 1);
-                const int64_t im = (int64_t)sc * W;   // the parent's Img row
-                int nimg = FG_AT(R.kped, sc, FG_N(int32_t, p.lay.rsize[RG_KPED])), e2 = FG_AT(R.klist, sc, FG_N(int32_t, p.lay.rsize[RG_KLIST]));
-                if (j < n2) {
-                    ++nimg;
+                nimg = warp_sum(nimg);
+                acc = warp_sum(acc) / 2;
+                for (int a = lane; a < nact; a += 32) {
+                    const int j = (int)FG_AT(R.act, a, FG_N(uint16_t, p.lay.rsize[RG_ACT]));
+                    if (j < n2 && ((FG_AT(imgw, im + j / WB, NIMGW) >> (j % WB)) & (Word)1)) continue;
+                    int e2 = acc;
 #pragma unroll
-                    for (int w = 0; w < W; ++w)
+                    for (int w = 0; w < W; ++w)   // none for the deletion's empty column
                         e2 += popcw((Word)(FG_AT(R.a2t, w * N2S + j, FG_N(Word, p.lay.rsize[RG_A2T])) &
-                                           FG_AT(imgc, im + w, NIMG)));
+                                           FG_AT(imgw, im + w, NIMGW)));
+                    const int d = succ_ped<W, Word>(p, R, V, B, s, j);
+                    const long long tt = (long long)d + (long long)c.vins * (n2 - nimg - (j < n2 ? 1 : 0)) +
+                                         (long long)c.eins * (m2.m - e2);
+                    const unsigned long long kk = ((unsigned long long)tt << 32) | (unsigned)d;
+                    const int cc = (s << kSelShift) | j;
+                    if (kk < key || (kk == key && cc < code)) {
+                        key = kk;
+                        code = cc;
+                    }
                 }
-                return (long long)ped_at(idx) + (long long)c.vins * (n2 - nimg) +
-                       (long long)c.eins * (m2.m - e2);
-            };
-            long long tmin = LLONG_MAX;
-            for (int k = lane; k < kw; k += 32) tmin = min(tmin, leaf_total(k));
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) tmin = min(tmin, (long long)__shfl_xor_sync(0xffffffffu, tmin, o));
-            if (lane == 0) FG_AT(S.wbest, warp, NSW) = (unsigned long long)tmin;
-            tm.sync();
-            long long best_total = LLONG_MAX;
-            for (int w = 0; w < NW; ++w) best_total = min(best_total, (long long)FG_AT(S.wbest, w, NSW));
-            tm.sync();
-            unsigned long long key = ~0ull;
-            for (int k = lane; k < kw; k += 32)
-                if (leaf_total(k) == best_total) {
-                    const unsigned long long kk =
-                        ((unsigned long long)ped_at(base + k) << 32) | (unsigned)(base + k);
-                    key = kk < key ? kk : key;
-                }
+            }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long y = __shfl_xor_sync(0xffffffffu, key, o);
-                key = y < key ? y : key;
+                const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, o);
+                const int c2 = __shfl_xor_sync(0xffffffffu, code, o);
+                if (k2 < key || (k2 == key && c2 < code)) {
+                    key = k2;
+                    code = c2;
+                }
             }
-            if (lane == 0) FG_AT(S.wbest, warp, NSW) = key;
+            if (lane == 0) {
+                FG_AT(S.wbest, warp, NSW) = key;
+                FG_AT(S.wcode, warp, NSW) = code;
+            }
             tm.sync();
-            unsigned long long bk = FG_AT(S.wbest, 0, NSW);
-            for (int w = 1; w < NW; ++w) bk = FG_AT(S.wbest, w, NSW) < bk ? FG_AT(S.wbest, w, NSW) : bk;
-            const int widx = (int)(bk & 0xffffffffull);
-            const int wv = decode(widx);
-            const int ws = wv >> kSelShift, wj = wv & ((1 << kSelShift) - 1);
-            int all = 0;
-            for (int w = 0; w < NW; ++w) all += FG_AT(S.wn, w, NSW);
+            key = FG_AT(S.wbest, 0, NSW);
+            code = FG_AT(S.wcode, 0, NSW);
+            for (int w = 1; w < NW; ++w) {
+                const unsigned long long k2 = FG_AT(S.wbest, w, NSW);
+                const int c2 = FG_AT(S.wcode, w, NSW);
+                if (k2 < key || (k2 == key && c2 < code)) {
+                    key = k2;
+                    code = c2;
+                }
+            }
+            const int ws = code >> kSelShift, wj = code & ((1 << kSelShift) - 1);
             if (tid == 0) {
-                FG_AT(p.out_cost, pair, p.n_pairs) = (int32_t)best_total;
-                if (p.out_nevals) FG_AT(p.out_nevals, pair, p.n_pairs) = nevals + 2LL * all;
+                FG_AT(p.out_cost, pair, p.n_pairs) = (int32_t)(key >> 32);
+                if (p.out_nevals) FG_AT(p.out_nevals, pair, p.n_pairs) = nevals + 2LL * total;
             }
             const int64_t mb = (int64_t)ws * (mrow / (int64_t)sizeof(MapT));   // the winner's map row
             const int64_t om = FG_AT(p.map_off, pair, p.n_pairs);
@@ -909,86 +1085,61 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
         }
 
         // ---- S4 selection ---------------------------------------------------------
-        // every warp reads the (bucket, warp) table: bucket totals, their exclusive prefix,
-        // and the bucket-b successors of the warps before this one; eight loads in flight
-        // per lane (a cluster team's table is in global scratch)
-        int tot = 0, mine = 0;
-        {
-            const int64_t hb = (int64_t)lane * NW;
-            int w = 0;
-            for (; w + 8 <= NW; w += 8) {
-                int v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = FG_AT(R.hist, hb + w + u, FG_N(int32_t, p.lay.rsize[RG_HIST]));
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    tot += v[u];
-                    mine += (w + u < warp) ? v[u] : 0;
-                }
-            }
-            for (; w < NW; ++w) {
-                const int v = FG_AT(R.hist, hb + w, FG_N(int32_t, p.lay.rsize[RG_HIST]));
-                tot += v;
-                mine += (w < warp) ? v : 0;
-            }
-        }
-        int incl = tot;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        const int bexcl = incl - tot;
-        int total = 0;   // successors of the level (the last bucket may hold padding)
-        for (int w = lane; w < NW; w += 32) total += FG_AT(S.wn, w, NSW);
-        total = warp_sum(total);
         const int newL = min(K, total);
-        // the bucket where the cumulative count reaches newL
-        const int thr = __ffs(__ballot_sync(0xffffffffu, bexcl < newL && incl >= newL)) - 1;
         if (tid == 0) nevals += total;
-        PHASE_MARK(2);
-        if (thr < hwin - 1) {
+        int thr, below, first;
+        find_threshold(p, htot, newL, thr, below, first);
+        const bool fits = A == A0 || first > 0;   // nothing below the anchor
+        rise = A - A0 + (first < kScoreMax ? first : kScoreMax);
+        if (fits && thr < kScoreMax && thr - first < hwin - 1) {
             // kept = every successor below the threshold bucket and the first q in it. Each
             // warp compacts its kept successors in enumeration order, then places them at
             // their rank in (PED, parent slot, j) order: position = #(smaller PED) +
-            // #(equal PED earlier); lane b holds the bucket-b counts of earlier warps.
-            const int q = newL - __shfl_sync(0xffffffffu, bexcl, thr);
-            const int eq_before = __shfl_sync(0xffffffffu, mine, thr);
-            const int lt_before = warp_sum(lane < thr ? mine : 0);
+            // #(equal PED earlier); lane b answers for bucket first + b.
+            const int q = newL - below;
+            const bool in = first + lane <= thr;
+            int incl = in ? FG_AT(htot, first + lane, kBuckets) : 0;
+            const int tot = incl;
+            const int mine = in ? FG_AT(hrow, first + lane, kBuckets) : 0;   // of earlier warps
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const int bexcl = incl - tot;
+            const int eq_before = __shfl_sync(0xffffffffu, mine, thr - first);
+            const int lt_before = warp_sum(first + lane < thr ? mine : 0);
             const int kbeg = lt_before + min(q, eq_before);
-            const int kcnt = compact_kept<Word>(p, R, base, kw, pa + thr, q, kbeg, eq_before, pk);
+            const int kcnt = compact_kept<Word>(p, R, V, thr, q, kbeg, eq_before);
             __syncwarp();
             PHASE_MARK(8);
-            int run = lane < thr ? mine : min(q, eq_before);   // kept of bucket `lane` before
+            // kept of bucket first + lane before the warp's next 32
+            int run = first + lane < thr ? mine : min(q, eq_before);
             for (int xb = 0; xb < kcnt; xb += 32) {
                 const int x = kbeg + xb + lane;
                 const bool v = xb + lane < kcnt;
-                const int d = v ? FG_AT(R.kped, x, FG_N(int32_t, p.lay.rsize[RG_KPED])) - pa : 0;
-                const unsigned V = __ballot_sync(0xffffffffu, v);
+                const int d = v ? FG_AT(R.kped, x, FG_N(int32_t, p.lay.rsize[RG_KPED])) - first : 0;
+                const unsigned V32 = __ballot_sync(0xffffffffu, v);
                 unsigned bb[5];
 #pragma unroll
                 for (int b = 0; b < 5; ++b) bb[b] = __ballot_sync(0xffffffffu, (d >> b) & 1);
                 const int pos = __shfl_sync(0xffffffffu, bexcl, d) +
                                 __shfl_sync(0xffffffffu, run, d) +
-                                __popc(same_value_lanes(V, bb, d) & lanemask_lt());
+                                __popc(same_value_lanes(V32, bb, d) & lanemask_lt());
                 if (v) {
-                    FG_AT(R.sel, pos, FG_N(int32_t, p.lay.rsize[RG_SEL])) = decode(FG_AT(R.klist, x, FG_N(int32_t, p.lay.rsize[RG_KLIST])));
-                    FG_AT(R.selped, pos, FG_N(int32_t, p.lay.rsize[RG_SELPED])) = d + pa;
+                    FG_AT(R.sel, pos, FG_N(int32_t, p.lay.rsize[RG_SEL])) = FG_AT(R.klist, x, FG_N(int32_t, p.lay.rsize[RG_KLIST]));
+                    FG_AT(R.selped, pos, FG_N(int32_t, p.lay.rsize[RG_SELPED])) = A + first + d;
                 }
-                unsigned m = V;
+                unsigned m = V32;
 #pragma unroll
                 for (int b = 0; b < 5; ++b) m &= ~(bb[b] ^ lanebit[b]);
                 run += __popc(m);
             }
             PHASE_MARK(9);
         } else {
-#ifdef FASTGED_PHASE_TIMERS
-            if (threadIdx.x == 0) ph[7] += 1;   // levels that took the exact selection
-#endif
-            select_exact<MapT, Word, CL, TS>(p, R.cand, R.klist, R.kped, R.sel, R.selped, S, L,
-                                             stride, newL, pa + hwin - 1, pk);
-            tm.sync();
-            for (int r = tid; r < newL; r += T) FG_AT(R.sel, r, FG_N(int32_t, p.lay.rsize[RG_SEL])) = decode(FG_AT(R.sel, r, FG_N(int32_t, p.lay.rsize[RG_SEL])));
+            const bool known = fits && thr < kScoreMax;
+            select_exact<W, Word, BK, CL>(p, R, V, B, n2, nw, newL, fits ? A : A0, known ? thr : -1, below);
+            PHASE_MARK(10);
         }
         tm.sync();
         PHASE_MARK(6);
@@ -1129,8 +1280,6 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
 #undef NP
 #undef NMAPT
 #undef NMAP16
-#undef NCK
-#undef NCK64
 #undef NIMGW
 }
 
@@ -1157,25 +1306,40 @@ __device__ __forceinline__ Regions<Word> make_regions(F base)
     R.img1 = (Word *)base(RG_IMG1);
     R.P = (Word *)base(RG_P);
     R.PL = (Word *)base(RG_PL);
-    R.cand = (int32_t *)base(RG_CAND);
+    R.score = base(RG_SCORE);
+    R.chist = (int32_t *)base(RG_CHIST);
     R.map0 = base(RG_MAP0);
     R.map1 = base(RG_MAP1);
     R.imgl = (Word *)base(RG_IMGL);
     return R;
 }
 
-// SM: every region lives in shared memory (addresses then stay in the shared window)
+// The regions that every layout keeps in shared memory: histogram rows, active columns and
+// their records, and the used-by-all mask. Taken from the shared window directly, their accesses (the
+// histogram's increments above all) need no generic addressing.
+template <typename Word>
+__device__ __forceinline__ void smem_regions(const KParams &p, Regions<Word> &R, uint8_t *smem)
+{
+    R.hist = (int32_t *)(smem + p.lay.off[RG_HIST]);
+    R.act = (uint16_t *)(smem + p.lay.off[RG_ACT]);
+    R.allm = (uint32_t *)(smem + p.lay.off[RG_ALL]);
+    R.rec = smem + p.lay.off[RG_REC];
+}
+
+// SM: every region but the neighbour lists and the vertex maps lives in shared memory (addresses then stay in the
+// shared window)
 template <int W, typename MapT, typename Word, bool SM, int BK>
-__global__ void __launch_bounds__(512, 2) kbest_kernel(const KParams p)
+__global__ void __launch_bounds__(512, (W <= 4) ? 2 : 1) kbest_kernel(const KParams p)
 {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ TeamShared S;
     uint8_t *gs = p.gscratch + (int64_t)blockIdx.x * p.lay.slice_bytes;
     auto base = [&](int r) -> uint8_t * {
-        if (SM) return smem + p.lay.off[r];
+        if (SM && r != RG_NBR && r != RG_MAP0 && r != RG_MAP1) return smem + p.lay.off[r];
         return ((p.lay.smem_mask >> r) & 1u ? smem : gs) + p.lay.off[r];
     };
-    const Regions<Word> R = make_regions<Word>(base);
+    Regions<Word> R = make_regions<Word>(base);
+    smem_regions(p, R, smem);
     for (;;) {
         if (threadIdx.x == 0) S.pair = atomicAdd(p.queue_head, 1);
         __syncthreads();
@@ -1202,7 +1366,8 @@ __global__ void __launch_bounds__(512, (W <= 2) ? 2 : 1) kbest_cluster_kernel(co
         if ((p.lay.smem_mask >> r) & 1u) return smem + p.lay.off[r];
         return ((p.lay.cta_mask >> r) & 1u ? gc : gs) + p.lay.off[r];
     };
-    const Regions<Word> R = make_regions<Word>(base);
+    Regions<Word> R = make_regions<Word>(base);
+    smem_regions(p, R, smem);
     TeamSharedCl &S = *(TeamSharedCl *)(gs + p.lay.team_off);
     for (;;) {
         if (crank == 0 && threadIdx.x == 0) S.pair = atomicAdd(p.queue_head, 1);

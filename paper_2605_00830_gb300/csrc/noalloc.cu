@@ -252,7 +252,7 @@ extern "C" int fastged_batch_noalloc(const fastged_cost_model *cost,
                         ? total
                         : std::min(max_dyn, (size_t)smem_per_sm / 2 - stat);
     plan_layout(cp, B, block, budget);
-    cp.all_smem = cp.lay.slice_bytes == 0 && kbest_has_smem_variant(cp.W, cp.wide, cp.w32);
+    cp.all_smem = layout_in_smem(cp.lay) && kbest_has_smem_variant(cp.W, cp.wide, cp.w32);
     int occ = 0;
     cudaError_t e = kbest_occupancy(cp.W, cp.wide, cp.w32, cp.all_smem, label_instance(B), block,
                                     (size_t)cp.lay.smem_bytes, &occ);
