@@ -40,6 +40,7 @@ enum Region : int {
     RG_HIST = 0, RG_ALPHA2, RG_A2T, RG_L2T, RG_SBASE, RG_PED0, RG_PED1, RG_SEL, RG_SELPED,
     RG_KLIST, RG_KPED, RG_NOFF, RG_NBR, RG_IMG0, RG_IMG1, RG_P, RG_PL,
     RG_SCORE, RG_MAP0, RG_MAP1, RG_IMGL, RG_CROW, RG_ACT, RG_ALL, RG_REC, RG_CHIST,
+    RG_ET0, RG_ET1,
     RG_COUNT
 };
 

@@ -413,7 +413,8 @@ void fastged::plan_layout(ClassPlan &cp, int B, int block, size_t budget)
     L.kmax = cp.kmax;
     L.n1max = cp.n1max;
     L.n2max = cp.n2max;
-    L.n2s = (int)align_up((size_t)std::max(cp.n2max, 1) + 1, 4);
+    // eight and more words: lanes take eight columns each (score_table)
+    L.n2s = (int)align_up((size_t)std::max(cp.n2max, 1) + 1, W >= 8 ? 8 : 4);
     L.mrow = (int)align_up((size_t)std::max(cp.n1max, 1) * msz, 16);
     L.word_bytes = (int)wb;
     L.B = B;
@@ -450,7 +451,9 @@ void fastged::plan_layout(ClassPlan &cp, int B, int block, size_t budget)
     sz[RG_PL] = (size_t)B * kl * W * wb;
     sz[RG_IMGL] = cp.cluster > 1 ? kl * W * wb : 0;
     // one byte per successor of the CTA's nodes
-    sz[RG_SCORE] = kl * (W == 1 ? ((cols / 4 - 1) | 1) * 4 : (size_t)cp.n2max + 1);
+    sz[RG_SCORE] = kl * (W == 1 ? ((cols / 4 - 1) | 1) * 4 : (size_t)L.n2s);
+    // the nodes' neighbour counts, two beam buffers
+    sz[RG_ET0] = sz[RG_ET1] = W >= 8 ? km * (size_t)L.n2s : 0;
     sz[RG_MAP0] = km * L.mrow;
     sz[RG_MAP1] = km * L.mrow;
     // shared memory is filled in order of access frequency; the rest goes to global scratch
@@ -459,14 +462,15 @@ void fastged::plan_layout(ClassPlan &cp, int B, int block, size_t budget)
     static const int prio[RG_COUNT] = {RG_HIST, RG_ACT, RG_ALL, RG_REC, RG_CROW, RG_ALPHA2, RG_SBASE,
                                        RG_PED0, RG_PED1, RG_SEL, RG_SELPED, RG_KLIST, RG_KPED,
                                        RG_NOFF, RG_A2T, RG_L2T, RG_IMG0, RG_IMG1, RG_P, RG_PL,
-                                       RG_SCORE, RG_NBR, RG_MAP0, RG_MAP1, RG_IMGL, RG_CHIST};
+                                       RG_SCORE, RG_NBR, RG_MAP0, RG_MAP1, RG_IMGL, RG_CHIST,
+                                       RG_ET0, RG_ET1};
     // cluster teams: the per-CTA tables the CTA writes (P, PL, sbase, staged Img) must be in
     // shared memory, so they come first
     static const int prio_cl[RG_COUNT] = {RG_HIST, RG_ACT, RG_ALL, RG_REC, RG_SBASE, RG_P, RG_PL,
                                           RG_IMGL, RG_CROW, RG_ALPHA2, RG_NOFF, RG_A2T, RG_L2T,
                                           RG_SCORE, RG_NBR, RG_CHIST, RG_PED0, RG_PED1, RG_SEL,
                                           RG_SELPED, RG_KLIST, RG_KPED, RG_IMG0, RG_IMG1,
-                                          RG_MAP0, RG_MAP1};
+                                          RG_MAP0, RG_MAP1, RG_ET0, RG_ET1};
     // a cluster team shares only global memory: its CTAs keep private shared-memory copies
     // of the read-only target-graph tables and neighbour lists, everything else is global
     auto cta_local = [](int r) {
@@ -781,21 +785,32 @@ static int tune_class(fastged_handle *h, ClassPlan &cp, int B, int forced_block,
         cap_grid(cp, max_sms, 1);
         return FASTGED_OK;
     }
-    int block = forced_block;
-    if (block == 0) block = cp.kmax <= 32 ? 128 : 256;
-    const size_t total = layout_total(cp, B, block);
-    size_t budget;
-    if (total + stat <= per_sm / 2 && total <= max_dyn) {
-        budget = total;                                   // all in shared memory
-    } else {
-        budget = std::min(max_dyn, per_sm / 2 - stat);    // keep two teams per SM
-    }
-    plan_layout(cp, B, block, budget);
-    cp.all_smem = layout_in_smem(cp.lay) && kbest_has_smem_variant(cp.W, cp.wide, cp.w32);
+    int block = forced_block ? forced_block : cp.kmax <= 32 ? 128 : 256;
     int occ = 0;
-    cudaError_t e = kbest_occupancy(cp.W, cp.wide, cp.w32, cp.all_smem, label_instance(B), block,
-                                    (size_t)cp.lay.smem_bytes, &occ);
+    auto plan = [&](int threads, int *teams) -> cudaError_t {
+        const size_t total = layout_total(cp, B, threads);
+        size_t budget;
+        if (total + stat <= per_sm / 2 && total <= max_dyn) {
+            budget = total;                                   // all in shared memory
+        } else {
+            budget = std::min(max_dyn, per_sm / 2 - stat);    // keep two teams per SM
+        }
+        plan_layout(cp, B, threads, budget);
+        cp.all_smem = layout_in_smem(cp.lay) && kbest_has_smem_variant(cp.W, cp.wide, cp.w32);
+        return kbest_occupancy(cp.W, cp.wide, cp.w32, cp.all_smem, label_instance(B), threads,
+                               (size_t)cp.lay.smem_bytes, teams);
+    };
+    cudaError_t e = plan(block, &occ);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
+    // where shared memory leaves two teams per SM, teams of 512 threads hide its latency, given
+    // a beam of 16 nodes per warp (1,024 dense pairs, K = 256: 19.6 -> 17.6 ms)
+    if (forced_block == 0 && block == 256 && occ == 2 && cp.kmax >= 256) {
+        int occ2 = 0;
+        e = plan(512, &occ2);
+        if (e == cudaSuccess && occ2 == 2) block = 512;
+        else e = plan(256, &occ);
+        if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
+    }
     if (occ < 1) return set_error(FASTGED_ERR_CUDA, "team does not fit on an SM");
     cp.block = block;
     cp.smem = (size_t)cp.lay.smem_bytes;

@@ -123,7 +123,7 @@ struct Regions {
     int32_t *ped0, *ped1;
     uint32_t *allm;
     uint16_t *act;
-    uint8_t *score, *rec;
+    uint8_t *score, *rec, *et0, *et1;
     Word *a2t, *l2t, *img0, *img1, *P, *PL, *imgl;
     uint8_t *map0, *map1;
 };
@@ -373,6 +373,106 @@ __device__ __forceinline__ void score_quads(const KParams &p, const Regions<Word
     }
 }
 
+// four bits of x (from bit 0) -> four bytes of 0 or 1
+__device__ __forceinline__ uint32_t nibble_bytes(uint32_t x)
+{
+    return ((x & 15u) * 0x00204081u) & 0x01010101u;
+}
+
+// Node vectors of a group in the lanes (lane t: node g0 + t) for score_table.
+struct TableNode {
+    int code;        // the node in the last level's selection: parent slot << kSelShift | j
+    int base;        // base PED less the anchor
+    int nimg;        // images in P
+    uint32_t ph[2];  // the first four prior neighbours' images, 16 bits each (0xffff: deleted)
+};
+
+// S3 over nodes [g0, g0 + ng) for targets of eight and more words and sparse, unlabelled pairs.
+// The implied edges of (s, j) need only two counts: E = g2 neighbours of j in Img(s), and T =
+// those in P(s). E differs from the parent's E by one row of A2, so each kept node keeps a row
+// of counts (a byte per column, double buffered): reading the parent's row, adding the bits
+// of A2[j_s] and writing it back replaces 2 W popcounts per column by about one addition, and
+// T is the sum of the bits of a few rows of A2 (deg of them).
+//   inserted = E - T, deleted = |P| - T, PED = base + C + eins (E - T) + edel (|P| - T)
+// Lanes <-> eight columns each (256 columns per step); the counts of four columns share a
+// 32-bit word, and no byte of E + |P| can pass 255 (the caller checks the degrees).
+template <int W, typename MapT, typename Word, bool FOLD>
+__device__ __forceinline__ void score_table(const KParams &p, const Regions<Word> &R,
+                                            const LevelView<Word> &V, int n2, int g0, int ng,
+                                            const TableNode &nd, const MapT *map, int64_t mt,
+                                            int n0, int deg, const uint8_t *ec, uint8_t *en,
+                                            bool root, int32_t *hrow)
+{
+    const int lane = threadIdx.x & 31;
+    const int N2S = p.lay.n2s;
+    const int c_eins = p.cost.eins, c_edel = p.cost.edel;
+    const uint8_t *a2b = (const uint8_t *)R.a2t, *imb = (const uint8_t *)V.imgw;
+    const int64_t NA = p.lay.rsize[RG_A2T], NE = p.lay.rsize[RG_ET0];
+    constexpr int WBY = (int)sizeof(Word);
+    for (int t = 0; t < ng; ++t) {
+        const int s = g0 + t;
+        const int code = __shfl_sync(0xffffffffu, nd.code, t);
+        const int np = __shfl_sync(0xffffffffu, nd.nimg, t);
+        const int base = __shfl_sync(0xffffffffu, nd.base, t) + (FOLD ? 0 : c_edel * np);
+        const uint32_t p0 = __shfl_sync(0xffffffffu, nd.ph[0], t), p1 = __shfl_sync(0xffffffffu, nd.ph[1], t);
+        const int par = code >> kSelShift, jc = code & ((1 << kSelShift) - 1);
+        for (int c0 = 8 * lane; c0 < V.stride; c0 += 256) {
+            const int wrow = (c0 / (8 * WBY)) * N2S, by = (c0 >> 3) % WBY;   // word row, byte in it
+            // bits c0 .. c0 + 7 of row u of A2 (columns and rows of A2 are alike; row n2 is empty)
+            // (columns past the last word: none)
+            const bool in = c0 < 8 * WBY * W;
+            auto bits = [&](int u) -> uint32_t {
+                return in ? (uint32_t)FG_AT(a2b, (int64_t)(wrow + u) * WBY + by, NA) : 0u;
+            };
+            uint32_t e[2] = {0u, 0u};
+            if (!root) {
+                const uint2 x = FG_AT((const uint2 *)ec, ((int64_t)par * N2S + c0) >> 3, NE >> 3);
+                const uint32_t a = bits(jc);
+                e[0] = x.x + nibble_bytes(a);
+                e[1] = x.y + nibble_bytes(a >> 4);
+            }
+            FG_AT((uint2 *)en, ((int64_t)s * N2S + c0) >> 3, NE >> 3) = make_uint2(e[0], e[1]);
+            uint32_t tt[2] = {0u, 0u};
+            auto image = [&](uint32_t u) {
+                if (u == 0xffffu) return;
+                const uint32_t a = bits((int)u);
+                tt[0] += nibble_bytes(a);
+                tt[1] += nibble_bytes(a >> 4);
+            };
+            if (deg > 0) image(p0 & 0xffffu);
+            if (deg > 1) image(p0 >> 16);
+            if (deg > 2) image(p1 & 0xffffu);
+            if (deg > 3) image(p1 >> 16);
+            for (int q = 4; q < deg; ++q) {
+                const int k = FG_AT(R.nbr, n0 + q, FG_N(int32_t, p.lay.rsize[RG_NBR])) & 0xffff;
+                image((uint32_t)FG_AT(map, (int64_t)s * mt + k, FG_N(MapT, p.lay.rsize[RG_MAP0])));
+            }
+            // used columns and the ones past the deletion
+            uint32_t um = c0 < n2 ? (uint32_t)FG_AT(imb, (int64_t)(s - V.ioff) * W * WBY + (c0 >> 3), V.nimg * WBY) : 0u;
+            if (c0 + 8 > n2 + 1) um |= c0 > n2 ? 0xffu : 0xffu << (n2 + 1 - c0);
+            uint32_t v4[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int4 cr = FG_AT((const int4 *)V.crow, (c0 >> 2) + h, N2S >> 2);
+                const int cw[4] = {cr.x, cr.y, cr.z, cr.w};
+                // FOLD: (E - T) + (|P| - T); else E - T, T apart
+                const uint32_t f = FOLD ? e[h] + (uint32_t)np * 0x01010101u - 2u * tt[h] : e[h] - tt[h];
+                v4[h] = 0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    int d = base + cw[u] + c_eins * (int)((f >> (8 * u)) & 0xffu);
+                    if (!FOLD) d -= c_edel * (int)((tt[h] >> (8 * u)) & 0xffu);
+                    int v = max(0, min(d, kScoreMax));
+                    if ((um >> (4 * h + u)) & 1u) v = kScoreMax;
+                    if (v < kScoreMax) atomicAdd(&FG_AT(hrow, v, kBuckets), 1);
+                    v4[h] |= (uint32_t)v << (8 * u);
+                }
+            }
+            FG_AT((uint2 *)R.score, ((int64_t)(s - V.cs0) * V.stride + c0) >> 3, FG_N(uint2, p.lay.rsize[RG_SCORE])) = make_uint2(v4[0], v4[1]);
+        }
+    }
+}
+
 // Scores this warp's nodes again for the exact selection (the node vectors are in place).
 template <int W, typename Word, int BK>
 __device__ __noinline__ void score_exact(const KParams &p, const Regions<Word> &R,
@@ -472,8 +572,9 @@ __device__ __forceinline__ void find_threshold(const KParams &p, const int32_t *
 
 // Stable compaction of this warp's kept successors, in enumeration order (the order of its
 // score bytes): every byte below `thr`, and the first q bytes equal to it counted over the
-// whole team. 16 bytes per lane and step. klist receives (parent slot << kSelShift) | j and
-// kped the byte, from position `pos`; eq: tied successors of the warps before this one.
+// whole team. 16 bytes per lane and step. klist receives the byte's index in the CTA's score
+// bytes (its node and column follow when all lanes have one to decode, in kept_code) and kped
+// the byte, from position `pos`; eq: tied successors of the warps before this one.
 template <typename Word>
 __device__ __forceinline__ int compact_kept(const KParams &p, const Regions<Word> &R,
                                             const LevelView<Word> &V, int thr, int q, int pos,
@@ -533,10 +634,7 @@ __device__ __forceinline__ int compact_kept(const KParams &p, const Regions<Word
                     m &= m - 1u;
                     const bool tie = (eqm[u] >> bit) & 1u;
                     if (tie && e++ >= q) continue;
-                    const uint32_t idx = (uint32_t)(o + 4 * u + (bit >> 3));
-                    const uint32_t row = idx / (uint32_t)V.stride;
-                    const int j = (int)FG_AT(R.act, idx - row * (uint32_t)V.stride, FG_N(uint16_t, p.lay.rsize[RG_ACT]));
-                    FG_AT(R.klist, at, FG_N(int32_t, p.lay.rsize[RG_KLIST])) = ((V.cs0 + (int)row) << kSelShift) | j;
+                    FG_AT(R.klist, at, FG_N(int32_t, p.lay.rsize[RG_KLIST])) = (int)(o + 4 * u + (bit >> 3));
                     FG_AT(R.kped, at, FG_N(int32_t, p.lay.rsize[RG_KPED])) = (int)((v[u] >> (bit & 24)) & 0xffu);
                     ++at;
                 }
@@ -547,6 +645,16 @@ __device__ __forceinline__ int compact_kept(const KParams &p, const Regions<Word
         eq += aeq;
     }
     return pos - pos0;
+}
+
+// (parent slot << kSelShift) | j of score byte idx.
+template <typename Word>
+__device__ __forceinline__ int kept_code(const KParams &p, const Regions<Word> &R,
+                                         const LevelView<Word> &V, int idx)
+{
+    const uint32_t row = (uint32_t)idx / (uint32_t)V.stride;
+    const int j = (int)FG_AT(R.act, (uint32_t)idx - row * (uint32_t)V.stride, FG_N(uint16_t, p.lay.rsize[RG_ACT]));
+    return ((V.cs0 + (int)row) << kSelShift) | j;
 }
 
 // Exact selection, used when the kept set reaches past the histogram window: the level is
@@ -599,7 +707,8 @@ __device__ __noinline__ void select_exact(const KParams &p, const Regions<Word> 
         const int kcnt = compact_kept<Word>(p, R, V, 1, q, kbeg, eq);
         __syncwarp();
         for (int x = kbeg + lane; x < kbeg + kcnt; x += 32) {
-            const int code = FG_AT(R.klist, x, NKL);
+            const int code = kept_code<Word>(p, R, V, FG_AT(R.klist, x, NKL));
+            FG_AT(R.klist, x, NKL) = code;
             FG_AT(R.kped, x, NKP) = succ_ped<W, Word>(p, R, V, B, code >> kSelShift, code & ((1 << kSelShift) - 1));
         }
     }
@@ -791,6 +900,23 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
     }
     // a pair without edge labels in a labelled batch pays nothing for the planes
     const int B = BK == 0 ? 0 : (__syncthreads_or(lab ? 1 : 0) ? Bc : 0);
+    // Neighbour counts kept per node (score_table): for eight and more words, without edge
+    // labels, when v_i has eight prior neighbours at most on average (each costs about one
+    // addition per column, the counts replace 2 W popcounts) and no count can pass 127.
+    bool table = false;
+    if (W >= 8) {
+        bool over = m1.m > 8 * n1;
+        for (int u = ltid; u < n2; u += LT) {
+            int d = 0;
+            for (int w = 0; w < nw; ++w) d += popcw(FG_AT(R.a2t, w * N2S + u, FG_N(Word, p.lay.rsize[RG_A2T])));
+            over |= d > 127;
+        }
+        for (int v = ltid; v < n1; v += LT)
+            over |= FG_AT(R.noff, v + 1, FG_N(int32_t, p.lay.rsize[RG_NOFF])) -
+                        FG_AT(R.noff, v, FG_N(int32_t, p.lay.rsize[RG_NOFF])) > 127;
+        table = !__syncthreads_or(over ? 1 : 0) && B == 0;
+    }
+    uint8_t *ecur = R.et0, *enext = R.et1;   // the parents' counts, and this level's
     long long nevals = 0;
     int L = 1, rise = 0;
     // current / next beam buffers, swapped after every level
@@ -839,6 +965,7 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
             }
 #pragma unroll
             for (int o = 16; o >= W32; o >>= 1) am &= __shfl_xor_sync(0xffffffffu, am, o);
+            if (table) am = 0u;   // rows of counts keep every column
             if (lane < W32) atomicAnd(&FG_AT(R.allm, lane, FG_N(uint32_t, p.lay.rsize[RG_ALL])), am);
         }
         __syncthreads();
@@ -877,7 +1004,7 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
                     }
                 }
             }
-            stride = nact;
+            stride = W >= 8 && table ? (nact + 7) / 8 * 8 : nact;
             // single-word rows: whole quads of columns, an odd number of them; the columns
             // past the active ones score past every bucket
             if (W == 1) {
@@ -919,6 +1046,7 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
             constexpr int NPL = BK == 8 ? kMaxB : (BK == 2 ? 2 : 1);
             Word pr = (Word)0, plr[NPL], imr = (Word)0;   // single-word node vectors
             int nbase = 0;
+            TableNode tn = {0, 0, 0, {0xffffffffu, 0xffffffffu}};
 #pragma unroll
             for (int b = 0; b < NPL; ++b) plr[b] = (Word)0;
             if (lane < ng) {
@@ -947,6 +1075,9 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
                     for (int u = 0; u < NU; ++u) {
                         const bool sub = phi[u] != DEL;
                         dcnt += (e[u] >= 0 && !sub) ? 1 : 0;
+                        if (W >= 8 && t0 == 0 && u < 4)
+                            tn.ph[u >> 1] = (tn.ph[u >> 1] & (u & 1 ? 0xffffu : 0xffff0000u)) |
+                                            (uint32_t)(uint16_t)phi[u] << (16 * (u & 1));
                         if (W == 1) {
                             const Word pb = sub ? (Word)1 << ((int)phi[u] % WB) : (Word)0;
                             pr |= pb;
@@ -976,6 +1107,11 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
                 for (int w = 0; w < W; ++w) used += popcw(FG_AT(imgw, im + w, NIMGW));
                 kw += n2 - used + 1;   // free g2 vertices (R_V2) and the deletion
                 if (W == 1) imr = FG_AT(imgw, im, NIMGW);
+                if (W >= 8 && table) {
+                    tn.code = i > 0 ? FG_AT(R.sel, s, FG_N(int32_t, p.lay.rsize[RG_SEL])) : 0;
+                    tn.base = nbase - A;
+                    tn.nimg = deg - dcnt;
+                }
             }
             __syncwarp();   // the group's node vectors (P, PL, base) are in place
             PHASE_MARK(5);
@@ -992,6 +1128,12 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
                 const int r = lane & ((1 << qs) - 1);
                 if (fold_ie) score_quads<Word, BK, true>(p, R, V, B, g0 + nd - cs0, nd < ng, r, qs, imr, pr, plr, nbase - A, hrow);
                 else score_quads<Word, BK, false>(p, R, V, B, g0 + nd - cs0, nd < ng, r, qs, imr, pr, plr, nbase - A, hrow);
+                PHASE_MARK(1);
+            } else if (W >= 8 && table && !last_b) {
+                const MapT *mp = (const MapT *)mapc;
+                const int64_t mt = mrow / (int64_t)sizeof(MapT);
+                if (fold_ie) score_table<W, MapT, Word, true>(p, R, V, n2, g0, ng, tn, mp, mt, n0, deg, ecur, enext, i == 0, hrow);
+                else score_table<W, MapT, Word, false>(p, R, V, n2, g0, ng, tn, mp, mt, n0, deg, ecur, enext, i == 0, hrow);
                 PHASE_MARK(1);
             } else if (!last_b) {
                 if (fold_ie) score_nodes<W, Word, BK, true, false>(p, R, V, B, n2, nw, g0, ng, A, 0, hrow);
@@ -1127,7 +1269,7 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
                                 __shfl_sync(0xffffffffu, run, d) +
                                 __popc(same_value_lanes(V32, bb, d) & lanemask_lt());
                 if (v) {
-                    FG_AT(R.sel, pos, FG_N(int32_t, p.lay.rsize[RG_SEL])) = FG_AT(R.klist, x, FG_N(int32_t, p.lay.rsize[RG_KLIST]));
+                    FG_AT(R.sel, pos, FG_N(int32_t, p.lay.rsize[RG_SEL])) = kept_code<Word>(p, R, V, FG_AT(R.klist, x, FG_N(int32_t, p.lay.rsize[RG_KLIST])));
                     FG_AT(R.selped, pos, FG_N(int32_t, p.lay.rsize[RG_SELPED])) = A + first + d;
                 }
                 unsigned m = V32;
@@ -1221,6 +1363,7 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
         PHASE_MARK(3);
         { int32_t *t = crc; crc = crn; crn = t; }
         { uint8_t *t = mapc; mapc = mapn; mapn = t; }
+        { uint8_t *t = ecur; ecur = enext; enext = t; }
         { Word *t = imgc; imgc = imgn; imgn = t; }
         { int32_t *t = pedc; pedc = pedn; pedn = t; }
         L = newL;
@@ -1307,6 +1450,8 @@ __device__ __forceinline__ Regions<Word> make_regions(F base)
     R.P = (Word *)base(RG_P);
     R.PL = (Word *)base(RG_PL);
     R.score = base(RG_SCORE);
+    R.et0 = base(RG_ET0);
+    R.et1 = base(RG_ET1);
     R.chist = (int32_t *)base(RG_CHIST);
     R.map0 = base(RG_MAP0);
     R.map1 = base(RG_MAP1);
