@@ -674,23 +674,28 @@ extern "C" void fastged_autotune_clear(void)
 }
 
 // A class whose pairs are fewer than the SMs may give each pair a cluster of CTAs: classes of
-// large graphs (four or more words), and two-word classes whose beam holds at least 2^16
-// successors per level.
+// large graphs (four or more words), and two-word classes whose beam holds at least 2^14
+// successors per level (one G(90, 0.4) pair, K = 500, 45,000 successors: 2.90 ms on one CTA).
 static bool cluster_eligible(const ClassPlan &cp, int npairs, int sm_count)
 {
     if (!kbest_has_cluster_variant(cp.W, cp.wide, cp.w32) || npairs >= sm_count) return false;
-    return cp.W >= 4 || (int64_t)cp.kmax * (cp.n2max + 1) >= 65536;
+    return cp.W >= 4 || (int64_t)cp.kmax * (cp.n2max + 1) >= 16384;
 }
 
-// CTAs per cluster without a tuning entry: about 20,000 successors of a level (K times the
-// target's vertices and the deletion) per CTA, between 2 and 8 CTAs (16 for a handful of
-// very wide pairs), then halved while the class's teams would take more than two waves of
-// the GPU (smaller teams spend fewer cluster barriers per successor).
+// CTAs per cluster without a tuning entry. A handful of pairs (16 CTAs each still fit the GPU
+// at once) takes 16: measured on 8 and 16 CTAs, one G(200, 0.4) pair 28.4 and 13.5 ms at
+// K = 5,000, 4.9 and 3.9 ms at K = 500; 4 pairs of 20 vertices 10.8 and 5.9 ms at K = 100,000;
+// 6 pairs of 700-1,000 vertices 76 and 45 ms at K = 1,024. Large graphs do so from 400,000
+// successors of a level (K times the target's vertices and the deletion) on; below, their
+// levels are too small (K = 32: 18.7 and 17.9 ms). Otherwise about 20,000 successors per CTA,
+// between 2 and 8 CTAs, halved while the class's teams would take more than two waves of the
+// GPU (smaller teams spend fewer cluster barriers per successor; 16 pairs at K = 100,000: 12.3
+// ms on 8 CTAs, 16.0 ms on 16).
 static int cluster_rule(const ClassPlan &cp, int npairs, int sm_count)
 {
     const int64_t succ = (int64_t)cp.kmax * (cp.n2max + 1);
+    if ((int64_t)npairs * 16 <= sm_count && succ >= (cp.W >= 8 ? 400000 : 16384)) return 16;
     int cl = succ <= 40000 ? 2 : succ <= 160000 ? 4 : 8;
-    if (succ >= 2000000 && (int64_t)npairs * 16 <= sm_count) cl = 16;
     while (cl > 2 && (int64_t)npairs * cl > 2 * (int64_t)sm_count) cl >>= 1;
     return cl;
 }
