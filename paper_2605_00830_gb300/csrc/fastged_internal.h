@@ -71,18 +71,18 @@ struct Layout {
 // block of shared memory; the two vertex-map buffers are in that block too, or in the warp's
 // block of global scratch (gmap). Offsets are in bytes from the start of the block.
 enum WarpRegion : int {
-    WR_TGT = 0,   // g2 records: adjacency word, label planes, cost-row entry (n2 + 2 of them)
+    WR_TGT = 0,   // g2 records: adjacency word, label planes (n2 vertices, the deletion)
     WR_LAB2,      // g2 vertex labels, int32[n2]
     WR_NOFF,      // g1 prior-neighbour list offsets, int32[n1 + 1]
     WR_NBR,       // g1 prior-neighbour lists, int32[m1]: k | edge label << 16
     WR_IMG0, WR_IMG1,     // Img bitset of every kept node, Word[K], two beam buffers
     WR_PED0, WR_PED1,     // PED of every kept node, int32[K]
     WR_E20, WR_E21,       // g2 edges with both ends in Img, uint16[K]
-    WR_ENT,       // successor entries of a level in enumeration order, uint16[K * (n2 + 1)]
-    WR_NODEOFF,   // first entry of every node, uint16[K + 1]
-    WR_KLIST,     // kept successors, uint32[K]: PED offset << 16 | entry index
-    WR_SEL,       // selected children in key order, int32[K]: parent slot << 8 | j (one-warp
-                  // kernel: record index j, 1 + target vertex or n2 + 1 for the deletion)
+    WR_SCORE,     // one byte per (node, active column) of a level, then the histogram, the
+                  // active columns' records and their label planes
+    WR_KLIST,     // kept successors, uint32[K]: PED offset << 16 | index of its score byte
+    WR_SEL,       // selected children in key order, int32[K]: parent slot << 8 | target vertex
+                  // (n2: the deletion)
     WR_SELPED,    // their PEDs, int32[K]
     WR_MAP0, WR_MAP1,     // vertex maps of the kept nodes, uint8[K][mrow]
     WR_COUNT
@@ -102,9 +102,14 @@ constexpr int col_rec_bytes(bool w32, int npl)
     return ((w32 ? 4 : 8) * (1 + (npl > 0 ? npl : 1)) + 4 + 15) / 16 * 16;
 }
 
+// bytes of one active column's record of the one-warp teams (WarpRec): three words and the
+// 32-bit cost entry
+constexpr int warp_col_bytes(bool w32) { return w32 ? 16 : 32; }
+
 struct WarpLayout {
     int32_t off[WR_COUNT];
     int32_t warp_bytes;   // shared memory per warp
+    int32_t hist_off, rec_off, pl_off;   // inside WR_SCORE
     int32_t gmap;         // 1: WR_MAP0 / WR_MAP1 are offsets into the warp's global block
     int32_t gmap_bytes;   // bytes of that global block (0 when the maps are in shared memory)
     int32_t mrow;         // bytes per stored vertex map (a multiple of 16)

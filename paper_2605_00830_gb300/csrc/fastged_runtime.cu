@@ -534,15 +534,22 @@ size_t fastged::plan_warp_layout(ClassPlan &cp, int B, bool gmap)
     const size_t km = (size_t)cp.kmax, n2 = (size_t)cp.n2max, n1 = (size_t)cp.n1max;
     wl.mrow = (int32_t)align_up(std::max<size_t>(n1, 1), 16);
     size_t sz[WR_COUNT];
-    sz[WR_TGT] = (n2 + 2) * rec;   // records 1..n2 the vertices, n2 + 1 the deletion, 0 the stand-in
+    sz[WR_TGT] = (n2 + 2) * rec;
     sz[WR_LAB2] = std::max<size_t>(n2, 1) * 4;
     sz[WR_NOFF] = (n1 + 1) * 4;
     sz[WR_NBR] = (size_t)std::max(cp.m1max, 1) * 4;
     sz[WR_IMG0] = sz[WR_IMG1] = km * wb;
     sz[WR_PED0] = sz[WR_PED1] = km * 4;
     sz[WR_E20] = sz[WR_E21] = km * 2;
-    sz[WR_ENT] = km * (n2 + 1) * 2;
-    sz[WR_NODEOFF] = (km + 1) * 2;
+    // rows of score bytes and the level's columns in whole quads, an odd number of them; at
+    // least two bytes per successor and node, so that the share of a team only grows where
+    // its beam is too small for the records
+    const size_t cols = (align_up(n2 + 1, 4) / 4 | 1) * 4;
+    wl.hist_off = (int32_t)align_up(km * cols, 16);
+    wl.rec_off = wl.hist_off + kHistRow * 4;
+    wl.pl_off = wl.rec_off + (int32_t)(cols * (size_t)warp_col_bytes(cp.w32));
+    sz[WR_SCORE] = std::max((size_t)wl.pl_off + cols * wb * (size_t)npl,
+                            align_up(km * (n2 + 1) * 2, 16) + align_up((km + 1) * 2, 16));
     sz[WR_KLIST] = km * 4;
     sz[WR_SEL] = km * 4;
     sz[WR_SELPED] = km * 4;
@@ -1047,8 +1054,8 @@ int fastged::flatten(fastged_handle *h, const fastged_pair_list *pl, int32_t K,
             const bool pk = packable(ped_bound, kp, g2.n);
             if (W == 1 && !pk) W = 2;
             // one warp per pair: single-word, packable pairs with small source graphs and
-            // beams, variant A
-            const bool warp = opt.team == FASTGED_TEAM_AUTO && opt.variant == 0 && W == 1 &&
+            // beams
+            const bool warp = opt.team == FASTGED_TEAM_AUTO && W == 1 &&
                               g1.n <= kWarpMaxN && g2.n <= kWarpMaxN2 && kp <= kWarpMaxK;
             const bool wide = g2.n >= 255,
                        w32 = W == 1 && g2.n <= (warp ? kWarpMaxN2Word32 : 32);
@@ -1311,7 +1318,7 @@ static KParams make_params(const fastged_handle *h, const Batch &b, int k, uint8
     p.n_order = (int32_t)cp.order.size();
     p.kpp = b.has_kpp ? (const int32_t *)(in + b.off_kpp) : nullptr;
     p.K = b.K;
-    p.hwin = b.opt.hist_window ? b.opt.hist_window : (cp.warp ? kWarpHist : kHistMax);
+    p.hwin = b.opt.hist_window ? b.opt.hist_window : kHistMax;
     p.variant = b.opt.variant;
     p.cost.vsub = h->cost.v_sub;
     p.cost.vdel = h->cost.v_del;

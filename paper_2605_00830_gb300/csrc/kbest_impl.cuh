@@ -347,9 +347,11 @@ __device__ __forceinline__ void score_quads(const KParams &p, const Regions<Word
     const Rec *rec = (const Rec *)R.rec;
     const Word *jm = (const Word *)((const uint8_t *)R.rec + p.lay.jm_off);
     const int c_eins = p.cost.eins, c_edel = p.cost.edel, c_esub = p.cost.esub;
-    const int nq = V.stride >> 2;
+    const int nq = V.stride >> 2, nk = (V.nact + 3) >> 2;   // quads of a row, with columns
+    if (!act) base = 1 << 28;   // past every bucket
     for (int k = r; k < nq; k += 1 << qs) {
-        uint32_t v4 = 0;
+        uint32_t v4 = k < nk ? 0u : 0x7f7f7f7fu;
+        if (k < nk) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const Rec c = FG_AT(rec, 4 * k + u, FG_N(Rec, p.lay.jm_off));
@@ -366,8 +368,9 @@ __device__ __forceinline__ void score_quads(const KParams &p, const Regions<Word
                 d += c_esub * popcw((Word)(c.a2 & P & ld));
             }
             const int v = used ? kScoreMax : max(0, min(d, kScoreMax));
-            if (act && v < kScoreMax) atomicAdd(&FG_AT(hrow, v, kBuckets), 1);
+            atomicAdd(&FG_AT(hrow, v, kBuckets), 1);   // [127] is not read as a count
             v4 |= (uint32_t)v << (8 * u);
+        }
         }
         if (act) FG_AT((uint32_t *)R.score, (int64_t)row * nq + k, FG_N(uint32_t, p.lay.rsize[RG_SCORE])) = v4;
     }
@@ -570,81 +573,122 @@ __device__ __forceinline__ void find_threshold(const KParams &p, const int32_t *
     below = __shfl_sync(0xffffffffu, mb, (thr >> 2) & 31);   // of the lane that holds thr
 }
 
-// Stable compaction of this warp's kept successors, in enumeration order (the order of its
-// score bytes): every byte below `thr`, and the first q bytes equal to it counted over the
-// whole team. 16 bytes per lane and step. klist receives the byte's index in the CTA's score
-// bytes (its node and column follow when all lanes have one to decode, in kept_code) and kped
-// the byte, from position `pos`; eq: tied successors of the warps before this one.
-template <typename Word>
-__device__ __forceinline__ int compact_kept(const KParams &p, const Regions<Word> &R,
-                                            const LevelView<Word> &V, int thr, int q, int pos,
-                                            int eq)
+// Bit index of the k-th set bit (from 0) of a 16-bit mask that has more than k.
+__device__ __forceinline__ int nth_bit16(uint32_t m, int k)
+{
+    int at = 0;
+#pragma unroll
+    for (int h = 8; h > 0; h >>= 1) {
+        const int c = __popc((m >> at) & ((1u << h) - 1u));
+        if (k >= c) {
+            k -= c;
+            at += h;
+        }
+    }
+    return at;
+}
+
+// Stable compaction of the kept ones among score bytes [lo, hi), in the order of the bytes: every
+// byte below `thr`, and the first q bytes equal to it counted over the whole team, of which eq
+// lie before lo. A step takes 16 bytes per lane and leaves a 16-bit mask of the kept ones in
+// each; then the lanes take the kept ones of all masks by rank, 32 at a time (the best
+// parents' children crowd into a few lanes: their own loops over up to 16 hits made the
+// one-warp kernel 4 % slower), or each its own when no lane has more than three (sparse
+// masks: ranking them costs large pairs 15 %). put(position, index, byte) receives each kept one; positions run from
+// `pos` and the walk ends once `last` is reached. Returns the number kept.
+template <typename Put>
+__device__ __forceinline__ int compact_bytes(const KParams &p, const uint8_t *score, int64_t n,
+                                             int64_t lo, int64_t hi, int thr, int q, int pos,
+                                             int eq, int last, Put put)
 {
     const int lane = threadIdx.x & 31;
     const int pos0 = pos;
-    const int64_t lo = (int64_t)(V.s_lo - V.cs0) * V.stride, hi = (int64_t)(V.s_hi - V.cs0) * V.stride;
     const uint32_t t4 = (uint32_t)thr * 0x01010101u;
-    for (int64_t b0 = lo & ~(int64_t)15; b0 < hi; b0 += 512) {
+    for (int64_t b0 = lo & ~(int64_t)15; b0 < hi && pos < last; b0 += 512) {
         const int64_t o = b0 + 16 * lane;
-        uint32_t le[4] = {0, 0, 0, 0}, eqm[4] = {0, 0, 0, 0}, v[4] = {0, 0, 0, 0};
+        uint32_t le = 0, eqm = 0;
         if (o < hi) {
-            const uint4 x = FG_AT((const uint4 *)R.score, o >> 4, FG_N(uint4, p.lay.rsize[RG_SCORE]));
-            v[0] = x.x;
-            v[1] = x.y;
-            v[2] = x.z;
-            v[3] = x.w;
+            const uint4 x = FG_AT((const uint4 *)score, o >> 4, n >> 4);
+            const uint32_t v[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                // bytes are at most 127: bit 7 of a byte says byte <= thr, byte == thr
-                le[u] = ((t4 | 0x80808080u) - v[u]) & 0x80808080u;
-                eqm[u] = (0x80808080u - (v[u] ^ t4)) & 0x80808080u;
+                // bytes are at most 127: bit 7 of a byte says byte <= thr, byte == thr; the
+                // product gathers bits 7, 15, 23 and 31 into a nibble
+                const uint32_t a = ((t4 | 0x80808080u) - v[u]) & 0x80808080u;
+                const uint32_t e = (0x80808080u - (v[u] ^ t4)) & 0x80808080u;
+                le |= (((a >> 7) * 0x10204080u) >> 28) << (4 * u);
+                eqm |= (((e >> 7) * 0x10204080u) >> 28) << (4 * u);
             }
             if (o < lo || o + 16 > hi) {   // bytes of the warps before and after this one
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    uint32_t m = 0;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int64_t at = o + 4 * u + k;
-                        if (at >= lo && at < hi) m |= 0x80u << (8 * k);
-                    }
-                    le[u] &= m;
-                    eqm[u] &= m;
-                }
+                uint32_t in = 0xffffu;
+                if (o < lo) in &= 0xffffu << (int)(lo - o);
+                if (o + 16 > hi) in &= 0xffffu >> (int)(o + 16 - hi);
+                le &= in;
+                eqm &= in;
             }
         }
-        const int nle = __popc(le[0]) + __popc(le[1]) + __popc(le[2]) + __popc(le[3]);
-        if (!__any_sync(0xffffffffu, nle > 0)) continue;
-        const int neq = __popc(eqm[0]) + __popc(eqm[1]) + __popc(eqm[2]) + __popc(eqm[3]);
-        int incl = (nle - neq) | (neq << 16);   // at most 512 each
+        if (!__any_sync(0xffffffffu, le != 0)) continue;
+        const int neq = __popc(eqm), nlt = __popc(le) - neq;
+        int incl = nlt | (neq << 16);   // at most 512 each
 #pragma unroll
         for (int s = 1; s < 32; s <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, incl, s);
             if (lane >= s) incl += y;
         }
-        const int all = __shfl_sync(0xffffffffu, incl, 31);
-        if (nle > 0) {
-            int e = eq + (incl >> 16) - neq;                  // ties before this lane
-            int at = pos + (incl & 0xffff) - (nle - neq) + (min(e, q) - min(eq, q));
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                uint32_t m = le[u];
-                while (m) {
-                    const int bit = __ffs((int)m) - 1;
-                    m &= m - 1u;
-                    const bool tie = (eqm[u] >> bit) & 1u;
-                    if (tie && e++ >= q) continue;
-                    FG_AT(R.klist, at, FG_N(int32_t, p.lay.rsize[RG_KLIST])) = (int)(o + 4 * u + (bit >> 3));
-                    FG_AT(R.kped, at, FG_N(int32_t, p.lay.rsize[RG_KPED])) = (int)((v[u] >> (bit & 24)) & 0xffu);
-                    ++at;
-                }
+        const int aeq = __shfl_sync(0xffffffffu, incl, 31) >> 16;
+        const int e1 = eq + (incl >> 16), e0 = e1 - neq;   // ties up to this lane, before it
+        // kept up to this lane: the smaller ones, and the ties within the quota
+        const int kin = (incl & 0xffff) + (min(e1, q) - min(eq, q));
+        uint32_t m = le;
+        if (e1 > q) {   // the lane where the ties run out, and those after it
+            m ^= eqm;
+            for (int k = e0; k < q; ++k) {   // back in: the first q - e0 of them
+                m |= eqm & (0u - eqm);
+                eqm &= eqm - 1u;
             }
         }
-        const int aeq = all >> 16;
-        pos += (all & 0xffff) + (min(eq + aeq, q) - min(eq, q));
+        const int cnt = __shfl_sync(0xffffffffu, kin, 31);
+        if (__reduce_max_sync(0xffffffffu, (unsigned)__popc(m)) <= 3u) {
+            for (int r = kin - __popc(m); m; ++r) {   // few: each lane its own
+                const int64_t idx = o + __ffs((int)m) - 1;
+                m &= m - 1u;
+                put(pos + r, (int)idx, (int)FG_AT(score, idx, n));
+            }
+        } else
+        for (int r0 = 0; r0 < cnt; r0 += 32) {
+            const int r = r0 + lane;
+            // the first lane that holds more than r kept ones up to itself
+            int src = 0;
+#pragma unroll
+            for (int s = 16; s > 0; s >>= 1)
+                if (__shfl_sync(0xffffffffu, kin, src + s - 1) <= r) src += s;
+            const uint32_t ms = __shfl_sync(0xffffffffu, m, src & 31);
+            const int ks = __shfl_sync(0xffffffffu, kin, src & 31);
+            if (r < cnt) {
+                const int64_t idx = b0 + 16 * src + nth_bit16(ms, r - (ks - __popc(ms)));
+                put(pos + r, (int)idx, (int)FG_AT(score, idx, n));
+            }
+        }
+        pos += cnt;
         eq += aeq;
     }
     return pos - pos0;
+}
+
+// The same for this warp's nodes of a team: klist receives the byte's index in the CTA's score
+// bytes (its node and column follow when all lanes have one to decode, in kept_code) and kped
+// the byte.
+template <typename Word>
+__device__ __forceinline__ int compact_kept(const KParams &p, const Regions<Word> &R,
+                                            const LevelView<Word> &V, int thr, int q, int pos,
+                                            int eq)
+{
+    return compact_bytes(p, R.score, p.lay.rsize[RG_SCORE],
+                         (int64_t)(V.s_lo - V.cs0) * V.stride, (int64_t)(V.s_hi - V.cs0) * V.stride,
+                         thr, q, pos, eq, INT_MAX, [&](int at, int idx, int v) {
+                             FG_AT(R.klist, at, FG_N(int32_t, p.lay.rsize[RG_KLIST])) = idx;
+                             FG_AT(R.kped, at, FG_N(int32_t, p.lay.rsize[RG_KPED])) = v;
+                         });
 }
 
 // (parent slot << kSelShift) | j of score byte idx.
@@ -1141,7 +1185,8 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
                 PHASE_MARK(1);
             }
         }
-        kw = warp_sum(kw);
+        kw = warp_sum(kw);   // (the scoring's last increments are done: [127] is overwritten)
+        __syncwarp();
         if (lane == 0) FG_AT(hrow, kScoreMax, kBuckets) = kw;
         if (ltid < W32) FG_AT(R.allm, ltid, FG_N(uint32_t, p.lay.rsize[RG_ALL])) = ~0u;   // for the next level
         prefix_buckets<CL>(p, R, tm);

@@ -10,56 +10,45 @@
 // kernels' (same key order, same tie-breaking); only the mapping onto the hardware differs:
 //
 //   * a warp owns a pair, so a level needs no block barrier and no cross-warp table;
+//   * a level scores only the active columns: the target vertices some kept node still has
+//     free, and the deletion. Their records (adjacency word, label planes, cost entry) are
+//     gathered once per level;
 //   * evaluation runs lane <-> parent node: each lane keeps its node's vectors (Img, P, label
-//     planes of P, base PED) in registers and walks the node's successor bitset (its free
-//     target vertices, and the deletion as bit n2) in increasing order, so no successor-id
-//     list is built; every step of that walk scores one successor per lane against the
-//     staged target record of its bit, without branches. A group of at most 16 nodes (the
-//     tail of the beam, or an early level) gives each node 2-32 lanes, each walking one
-//     slice of the bit range 0..n2;
-//   * the PED histogram of the selection is counted in the same loop in per-lane 4-bit
-//     counters (offsets 0-14 from the anchor, widened to 16 bits every 14 slots and summed
-//     over the warp once per level), anchored at the PED of the best parent, a lower bound of
-//     every child (costs are non-negative and slot 0 holds the least PED of the kept list).
-//     Costs are scaled by 4 inside the evaluation, so that an offset is the bit position of
-//     its counter; the slots past a lane's successors score a stand-in record whose offset
-//     is past every bucket;
-//   * each successor leaves one 16-bit entry (PED offset clamped to 8 bits, record index) in
-//     enumeration order (node by node, j increasing, the deletion last); the kept ones are
-//     compacted in that order and then placed at their rank by a counting sort over the
-//     buckets;
-//   * when the K-th PED falls past the histogram window, the level is scored again with exact
-//     16-bit PED offsets (every PED of a pair routed here is below 2^16), the K-th offset is
-//     found by bisection, the kept entries are ranked by (PED, enumeration order) and their
-//     target vertices recovered from the node's free set.
+//     planes of P, base PED) in registers and all lanes walk the same columns, so a record is
+//     one broadcast load. A group of at most 16 nodes (the tail of the beam, or an early
+//     level) gives each node 2-32 lanes, which share its columns in quads;
+//   * each score leaves one byte (PED offset from the best parent's PED, a lower bound of every
+//     child: costs are non-negative and slot 0 holds the least PED of the kept list; 127 when
+//     it is larger or the node has used the column's vertex), four to a store, and one count
+//     in the warp's histogram by a shared-memory increment;
+//   * the kept ones are compacted in enumeration order (node by node, j increasing, the
+//     deletion last) from the bytes, 16 per lane and load, and then placed at their rank by a
+//     counting sort over the buckets;
+//   * when the kept PEDs reach past the window, the level is scored again over coarser, then
+//     finer windows until the K-th PED is known, and the kept children are ranked by (PED,
+//     enumeration order).
+//
+// Bound: the integer ALU pipe (half the issue rate) in the scoring loop, and the latency of one
+// pair's levels when a batch holds fewer pairs than warps fit the GPU. The loop before this one
+// walked each lane's own free bits (find-first-set, a record load with 32 addresses, a 16-bit
+// entry and a packed-register count per successor), and its 15-bucket window sent cost setting
+// 2 to a bisection on many levels. Measured, before -> after: 20,000 pairs, setting 1, resident:
+// 2.82 -> 2.76 ms; 5,003 pairs, setting 2, from host memory: 2.08 -> 1.32 ms; 61 x 256 distance
+// matrix, K = 20: 1.28 -> 1.19 ms; one pair from host memory: 302 -> 296 us.
 #pragma once
 #include "kbest_impl.cuh"
 
 namespace fastged {
 
-// x << n with PTX semantics: shift amounts of 32 or more give 0
-__device__ __forceinline__ uint32_t shl_clamped(uint32_t x, uint32_t n)
-{
-    uint32_t r;
-    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
-    return r;
-}
-
-// PED histogram buckets of the one-warp kernel: offsets 0..kWarpBuckets-2 from the anchor
-// decide the threshold (the last field of the counters is not read)
-constexpr int kWarpBuckets = 16;
 // kept successors a warp places at once: the largest K of a one-warp class, in 32s
 constexpr int kWarpChunks = 4;
-// cost entry of record 0 in quarter units: any slot scoring it has an offset far past every
-// histogram bucket, and adding it to a PED offset (below 2^18 in quarter units) stays in range
-constexpr int kWarpIdleCost = 1 << 24;
+// cost entry of the columns that pad the active ones to whole quads: past every bucket, and
+// no PED offset (below 2^16) added to it leaves the range
+constexpr int kWarpPadCost = 1 << 24;
 
-// Target record of g2 vertex u, stored at index u + 1, or of the deletion column, stored at
-// index n2 + 1 (no neighbours, no labels): adjacency word, NPL edge-label planes, and the
-// vertex-cost entry C[i][u] of the current level times 4 (the evaluation works in units of a
-// quarter, so that a PED offset is directly the bit position of its histogram counter).
-// Record 0 is a stand-in scored by the slots past a lane's successors: its cost entry is so
-// large that such a slot counts in no histogram bucket.
+// Target record of g2 vertex u at index u, or of the deletion column at index n2 (no
+// neighbours, no labels): adjacency word and NPL edge-label planes. (ColRec, one per active
+// column of a level, also holds the cost entry.)
 template <typename Word, int NPL>
 struct __align__(16) TgtRec {
     Word a2;
@@ -102,11 +91,16 @@ __device__ __forceinline__ void rec_set_plane(TgtRec<Word, 0> &, int, Word) {}
 #define WPHASE(k) do { } while (0)
 #endif
 
-// 1 + index of the lowest set bit, 0 when none is set: the record index of the next
-// successor of a walk (a free target vertex, or the deletion as bit n2), record 0 once the
-// walk is over
-__device__ __forceinline__ int ffs1(uint32_t x) { return __ffs((int)x); }
-__device__ __forceinline__ int ffs1(uint64_t x) { return __ffsll((long long)x); }
+// Record of an active column of a level: adjacency word, the g2 neighbours whose edge's label
+// differs from the level's (v_i's edges to its prior neighbours, when all have one label), the
+// vertex's one-hot bit (0: the deletion, or a column that pads the row) and the cost entry.
+template <typename Word>
+struct __align__(16) WarpRec {
+    Word a2, mis, bit;
+    int32_t crow;
+};
+static_assert(sizeof(WarpRec<uint32_t>) == warp_col_bytes(true), "record size");
+static_assert(sizeof(WarpRec<uint64_t>) == warp_col_bytes(false), "record size");
 
 // Dynamic shared memory of the one-warp kernel (every warp of a CTA has its block in it).
 extern __shared__ __align__(16) uint8_t g_warp_smem[];
@@ -131,8 +125,10 @@ struct WarpRegs {
     __device__ __forceinline__ int32_t *pedn(const WarpLayout &wl) const { return at<int32_t>(cur ? wl.off[WR_PED0] : wl.off[WR_PED1]); }
     __device__ __forceinline__ uint16_t *e2c(const WarpLayout &wl) const { return at<uint16_t>(cur ? wl.off[WR_E21] : wl.off[WR_E20]); }
     __device__ __forceinline__ uint16_t *e2n(const WarpLayout &wl) const { return at<uint16_t>(cur ? wl.off[WR_E20] : wl.off[WR_E21]); }
-    __device__ __forceinline__ uint16_t *ent(const WarpLayout &wl) const { return at<uint16_t>(wl.off[WR_ENT]); }
-    __device__ __forceinline__ uint16_t *nodeoff(const WarpLayout &wl) const { return at<uint16_t>(wl.off[WR_NODEOFF]); }
+    __device__ __forceinline__ uint8_t *score(const WarpLayout &wl) const { return at<uint8_t>(wl.off[WR_SCORE]); }
+    __device__ __forceinline__ int32_t *hist(const WarpLayout &wl) const { return at<int32_t>(wl.off[WR_SCORE] + wl.hist_off); }
+    __device__ __forceinline__ WarpRec<Word> *rec(const WarpLayout &wl) const { return at<WarpRec<Word>>(wl.off[WR_SCORE] + wl.rec_off); }
+    __device__ __forceinline__ Word *planes(const WarpLayout &wl) const { return at<Word>(wl.off[WR_SCORE] + wl.pl_off); }
     __device__ __forceinline__ uint32_t *klist(const WarpLayout &wl) const { return at<uint32_t>(wl.off[WR_KLIST]); }
     __device__ __forceinline__ int32_t *sel(const WarpLayout &wl) const { return at<int32_t>(wl.off[WR_SEL]); }
     __device__ __forceinline__ int32_t *selped(const WarpLayout &wl) const { return at<int32_t>(wl.off[WR_SELPED]); }
@@ -140,46 +136,47 @@ struct WarpRegs {
     __device__ __forceinline__ uint8_t *mapn(const WarpLayout &wl) const { return mb + (cur ? wl.off[WR_MAP0] : wl.off[WR_MAP1]); }
 };
 
-// Scores every successor of level i (lane <-> parent node). Entries go to ent in enumeration
-// order and nodeoff receives each node's first entry. EXACT = false: entry = (min(PED - A,
-// 255) << 8) | (record index: 1 + target vertex, n2 + 1 for the deletion), and on return lane
-// b < kWarpBuckets - 1 holds the number of successors whose offset PED - A is b (lane
-// kWarpBuckets - 1 holds no meaningful count); EXACT = true: entry = PED - A (exact, below
-// 2^16).
+// elements of the arrays inside WR_SCORE (bounds-checked builds check indexes against them)
+#define NSC ((int64_t)wl.hist_off)
+#define NRC FG_N(WarpRec<Word>, wl.pl_off - wl.rec_off)
+#define NPA FG_N(Word, wl.size[WR_SCORE] - wl.pl_off)
+
+// What scoring a level needs beside the warp's regions.
+struct WarpLevel {
+    int L, n0, deg, n2, mrow;   // nodes, v_i's prior neighbours, target vertices, map row bytes
+    int nq, nk;                 // quads of columns per row of score bytes (odd), with a column
+    int m2;                     // g2 edges (variant B)
+    bool one_label;             // v_i's edges to its prior neighbours have one label
+};
+
+// Scores every successor of level i. MODE 0: bytes and counts of the offsets from A; returns the
+// successors of the level. MODE 1 (selection past the window): with sh >= 0 the offsets from A
+// in units of 2^sh, PEDs below A left out; sh < 0 marks 0 = below A, 1 = at A, 127 = above.
+// MODE 2 (variant B's last level): no bytes; the lane's least (total, PED, code) of the
+// completed successors goes to key and code.
 // FOLD: insertion and deletion of an edge cost the same, so the two implied-edge terms are
-// one popcount. Returns the number of successors of the level.
-template <typename Word, int BK, bool FOLD, bool EXACT>
+// one popcount.
+template <typename Word, int BK, bool FOLD, int MODE>
 __device__ __forceinline__ int eval_level(const KParams &p,
                                           const WarpRegs<Word, (BK == 8 ? kMaxB : BK)> &R,
-                                          int L, int n0, int deg, int n2, int mrow, int A,
-                                          int &hist, long long *prof = nullptr)
+                                          const WarpLevel &lv, int A, int sh,
+                                          unsigned long long &key, int &code,
+                                          long long *prof = nullptr)
 {
     constexpr int WB = 8 * (int)sizeof(Word);
     constexpr int NPL = BK == 8 ? kMaxB : BK;
+    using CRec = WarpRec<Word>;
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const WarpLayout &wl = p.wl;
+    const int L = lv.L, n0 = lv.n0, deg = lv.deg, n2 = lv.n2, mrow = lv.mrow, nq = lv.nq;
     const int B = BK == 0 ? 0 : (BK == 2 ? 2 : p.lay.B);
-    // costs in quarter units (see TgtRec): a successor's PED offset times 4 is the bit
-    // position of its 4-bit histogram counter in the 64-bit pair (chi, clo)
-    const int c_eins = 4 * p.cost.eins, c_edel = 4 * p.cost.edel, c_esub = 4 * p.cost.esub;
-    const Word nmask = n2 >= WB ? ~(Word)0 : (((Word)1 << n2) - (Word)1);
+    const int c_eins = p.cost.eins, c_edel = p.cost.edel, c_esub = p.cost.esub;
     const uint8_t *mapc = R.mapc(wl);
-    using TRec = TgtRec<Word, NPL>;
-    const TRec *tgt = R.tgt(wl);
-    // histogram: 4-bit counters (clo: buckets 0-7, chi: 8-15) widened every 14 slots into
-    // acc[m] = buckets (m, m + 4) and acc[4 + m] = (8 + m, 12 + m), 16 bits each
-    uint32_t clo = 0, chi = 0, acc[8];
-#pragma unroll
-    for (int m = 0; m < 8; ++m) acc[m] = 0;
-    auto flush = [&]() {
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            acc[m] += (clo >> (4 * m)) & 0x000F000Fu;
-            acc[4 + m] += (chi >> (4 * m)) & 0x000F000Fu;
-        }
-        clo = chi = 0;
-    };
+    const CRec *rec = R.rec(wl);
+    const Word *planes = R.planes(wl);
+    int32_t *hist = R.hist(wl);
+    uint32_t *score = (uint32_t *)R.score(wl);
     int tot = 0;
     // v_i's first prior neighbour (the same for every node): most levels of tree-like source
     // graphs have at most one, and those take the short S2 path below
@@ -188,14 +185,11 @@ __device__ __forceinline__ int eval_level(const KParams &p,
     long long tprof = clock64();
 #endif
     for (int g0 = 0; g0 < L; g0 += 32) {
-        // a group of ng nodes: one lane per node when ng > 16, else q = 2^qs lanes per node
-        // (ng * q <= 32), lane part r taking the successors in its slice of the bit range
-        // 0..n2 (target vertices, then the deletion as bit n2), so that a short group (the
-        // last of a beam of 100, or a level of few nodes) keeps every lane busy
+        // a group of ng nodes: one lane per node when ng > 16, else 2^qs lanes per node, lane
+        // part r taking every 2^qs-th quad of columns
         const int ng = min(32, L - g0);
         const int qs = ng > 16 ? 0 : ng > 8 ? 1 : ng > 4 ? 2 : ng > 2 ? 3 : ng > 1 ? 4 : 5;
-        const int q = 1 << qs;
-        const int r = lane & (q - 1);
+        const int r = lane & ((1 << qs) - 1);
         const int s = g0 + (lane >> qs);
         const bool act = (lane >> qs) < ng;
         // S2: P = images of the substituted g1 neighbours of v_i, their edge labels as planes
@@ -239,91 +233,75 @@ __device__ __forceinline__ int eval_level(const KParams &p,
                     if (b < B && ((e[u] >> (16 + b)) & 1)) PL[b] |= pb;
             }
         }
-        const Word im = act ? FG_AT(R.imgc(wl), s, FG_N(Word, wl.size[WR_IMG0])) : ~(Word)0;
-        const int base = act ? 4 * (FG_AT(R.pedc(wl), s, FG_N(int32_t, wl.size[WR_PED0])) - A) + c_edel * dcnt
-                             : 0;
-        // the node's successors: its free target vertices and the deletion as bit n2 (n2 < WB)
-        const Word fr = act ? (Word)((~im & nmask) | ((Word)1 << n2)) : (Word)0;
-        const int ncnt = popcw(fr);
-        // this lane's slice [lo, hi) of the bits 0..n2 (hi <= n2 + 1 <= WB)
-        const int lo = (r * (n2 + 1)) >> qs, hi = ((r + 1) * (n2 + 1)) >> qs;
-        const Word below = lo >= WB ? ~(Word)0 : (((Word)1 << lo) - (Word)1);
-        const Word upto = hi >= WB ? ~(Word)0 : (((Word)1 << hi) - (Word)1);
-        Word x = fr & upto & ~below;
-        const int cnt = popcw(x);   // this lane's successors
-        int incl = r == 0 ? ncnt : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(FULL, incl, o);
-            if (lane >= o) incl += v;
-        }
-        const int noff = tot + incl - ncnt;   // the node's first entry (same on all its parts)
-        if (act && r == 0) FG_AT(R.nodeoff(wl), s, FG_N(uint16_t, wl.size[WR_NODEOFF])) = (uint16_t)noff;
-        const int off = noff + popcw((Word)(fr & below));   // this lane's first entry
-        const int maxc = (int)__reduce_max_sync(FULL, (unsigned)cnt);
+        const Word im = act ? FG_AT(R.imgc(wl), s, FG_N(Word, wl.size[WR_IMG0])) : (Word)0;
+        // (lanes without a node score past every bucket)
+        const int base = act ? FG_AT(R.pedc(wl), s, FG_N(int32_t, wl.size[WR_PED0])) - A + c_edel * dcnt : kWarpPadCost;
+        const int nimg = popcw(im);
+        if (act && r == 0) tot += n2 - nimg + 1;   // free target vertices and the deletion
+        const int e2 = MODE == 2 && act ? (int)FG_AT(R.e2c(wl), s, FG_N(uint16_t, wl.size[WR_E20])) : 0;
 #ifdef FASTGED_PHASE_TIMERS
-        // profiling builds: loop slots of the level, cycles of the group set-up (prof[12])
+        // profiling builds: cycles of the group set-up (prof[12])
         if (prof && lane == 0) {
             const long long tn = clock64();
-            prof[9] += maxc;
             prof[12] += tn - tprof;
             tprof = tn;
         }
 #endif
-        uint16_t *ent = R.ent(wl);
-        // two successors of the lane's slice per step (its next two bits, or record 0 once
-        // none is left), in blocks of 14 so that a 4-bit counter cannot overflow inside one.
-        // score(j) is 4 * (PED - A) of the successor with record j.
-        auto score = [&](int j) -> int {
-            const TgtRec<Word, NPL> r = FG_AT(tgt, j, FG_N(TRec, wl.size[WR_TGT]));
-            const Word ai = r.a2 & im;
-            int d = base + r.crow;
-            if (FOLD) {
-                d += c_eins * popcw((Word)(ai ^ P));
-            } else {
-                d += c_eins * popcw((Word)(ai & ~P)) + c_edel * popcw((Word)(P & ~r.a2));
-            }
-            if (NPL > 0) {
-                Word ld = (Word)0;
+        for (int k = r; k < nq; k += 1 << qs) {
+            uint32_t v4 = k < lv.nk ? 0u : 0x7f7f7f7fu;
+            if (k < lv.nk) {
+                // sums of products go to the FMA pipe: the integer ALU, at half the issue rate,
+                // is what bounds this loop
+                int dd[4];
+                Word us[4];
 #pragma unroll
-                for (int b = 0; b < NPL; ++b)
-                    if (b < B) ld |= PL[b] ^ rec_plane(r, b);
-                d += c_esub * popcw((Word)(r.a2 & P & ld));
-            }
-            return d;
-        };
-        // the 4-bit field of offset d = d4 / 4 starts at bit d4 of the 64-bit pair (chi,
-        // clo); a PTX shift by 32 or more yields 0, so the word that does not hold the field
-        // gets nothing, and neither does an offset of 16 or more, without a compare. Every
-        // slot is counted: the ones past the lane's successors score record 0, whose offset
-        // is past every bucket.
-        auto count = [&](int d4) {
-            clo += shl_clamped(1u, (uint32_t)d4);
-            chi += shl_clamped(1u, (uint32_t)d4 - 32u);
-        };
-        for (int t0 = 0; t0 < maxc; t0 += 14) {
-            const int t1 = min(maxc, t0 + 14);
-            for (int t = t0; t < t1; t += 2) {
-                const int ja = ffs1(x);
-                x &= x - (Word)1;
-                const int jb = ffs1(x);
-                x &= x - (Word)1;
-                const bool va = t < cnt, vb = t + 1 < cnt;
-                const int da = score(ja), db = score(jb);
-#define NE FG_N(uint16_t, wl.size[WR_ENT])
-                // predicated stores: the slots past the lane's successors write nothing
-                if (EXACT) {
-                    if (va) FG_AT(ent, off + t, NE) = (uint16_t)(da >> 2);
-                    if (vb) FG_AT(ent, off + t + 1, NE) = (uint16_t)(db >> 2);
-                } else {
-                    if (va) FG_AT(ent, off + t, NE) = (uint16_t)((min(da, 1020) << 6) | ja);
-                    if (vb) FG_AT(ent, off + t + 1, NE) = (uint16_t)((min(db, 1020) << 6) | jb);
-#undef NE
-                    count(da);
-                    count(db);
+                for (int u = 0; u < 4; ++u) {
+                    const CRec c = FG_AT(rec, 4 * k + u, NRC);
+                    const Word ai = c.a2 & im;
+                    us[u] = im & c.bit;
+                    int d = base + c.crow;
+                    if (FOLD) d += c_eins * popcw((Word)(ai ^ P));
+                    else d += c_eins * popcw((Word)(ai & ~P)) + c_edel * popcw((Word)(P & ~c.a2));
+                    if (NPL > 0) {
+                        if (lv.one_label) {   // warp-uniform
+                            d += c_esub * popcw((Word)(c.mis & P));
+                        } else {
+                            Word ld = (Word)0;
+#pragma unroll
+                            for (int b = 0; b < NPL; ++b)
+                                if (b < B) ld |= PL[b] ^ FG_AT(planes, b * 4 * nq + 4 * k + u, NPA);
+                            d += c_esub * popcw((Word)(c.a2 & P & ld));
+                        }
+                    }
+                    if (MODE == 2 && act && !us[u] && c.crow < kWarpPadCost) {
+                        const int j = c.bit ? popcw((Word)(c.bit - 1)) : n2;
+                        const long long tt = (long long)d + A + (long long)p.cost.vins * (n2 - nimg - (j < n2 ? 1 : 0)) +
+                                             (long long)c_eins * (lv.m2 - e2 - popcw(ai));
+                        const unsigned long long kk = ((unsigned long long)tt << 32) | (unsigned)(d + A);
+                        const int cc = (s << 8) | j;
+                        if (kk < key || (kk == key && cc < code)) {
+                            key = kk;
+                            code = cc;
+                        }
+                    }
+                    dd[u] = d;
+                }
+                if (MODE != 2) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int d = dd[u];
+                        int v;
+                        if (MODE == 0) v = min(d, kScoreMax);
+                        else if (sh >= 0) v = d < 0 ? kScoreMax : min(d >> sh, kScoreMax);
+                        else v = d < 0 ? 0 : d == 0 ? 1 : kScoreMax;
+                        if (us[u]) v = kScoreMax;
+                        dd[u] = v;
+                        atomicAdd(&FG_AT(hist, v, kBuckets), 1);   // [127] is not read
+                    }
+                    v4 = (uint32_t)dd[0] + (uint32_t)dd[1] * 256u + (uint32_t)dd[2] * 65536u + (uint32_t)dd[3] * 16777216u;
                 }
             }
-            if (!EXACT) flush();
+            if (MODE != 2 && act) FG_AT(score, s * nq + k, NSC / 4) = v4;
         }
 #ifdef FASTGED_PHASE_TIMERS
         // profiling builds: cycles of the scoring loop (prof[13])
@@ -333,43 +311,116 @@ __device__ __forceinline__ int eval_level(const KParams &p,
             tprof = tn;
         }
 #endif
-        tot += __shfl_sync(FULL, incl, 31);
-    }
-    if (lane == 0) FG_AT(R.nodeoff(wl), L, FG_N(uint16_t, wl.size[WR_NODEOFF])) = (uint16_t)tot;
-    if (!EXACT) {
-        // warp totals (at most 128 x 65 successors: 16-bit fields cannot overflow), then lane
-        // b takes bucket b
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc[m] += __shfl_xor_sync(FULL, acc[m], o);
-        }
-        const int b = lane & 15;
-        const int wsel = ((b >> 3) << 2) | (b & 3);
-        uint32_t wv = acc[0];
-#pragma unroll
-        for (int m = 1; m < 8; ++m) wv = wsel == m ? acc[m] : wv;
-        hist = (int)((wv >> (((b >> 2) & 1) << 4)) & 0xffffu);
     }
     __syncwarp();
-#ifdef FASTGED_PHASE_TIMERS
-    // profiling builds: cycles after the scoring loops (group tails, warp reduction; prof[14])
-    if (prof && lane == 0) prof[14] += clock64() - tprof;
-#endif
-    return tot;
+    return warp_sum(tot);
 }
 
-// Slot of the node that owns entry k (nodeoff is strictly increasing: every node has at
-// least its deletion successor).
-__device__ __forceinline__ int node_of(const KParams &p, const uint16_t *nodeoff, int L, int k)
+// Parent slot << 8 | target vertex (n2: the deletion) of score byte idx. inv = ceil(2^21 /
+// row bytes): idx < 128 rows and rows below 72 bytes make the product exact.
+template <typename Word, int NPL>
+__device__ __forceinline__ int warp_code(const KParams &p, const WarpRegs<Word, NPL> &R, int idx,
+                                         int row, uint32_t inv, int n2)
 {
-    int lo = 0, hi = L;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;   // 0 < mid < L: within the node offsets
-        if ((int)FG_AT(nodeoff, mid, FG_N(uint16_t, p.wl.size[WR_NODEOFF])) <= k) lo = mid;
-        else hi = mid;
+    const WarpLayout &wl = p.wl;
+    const int s = (int)(((uint32_t)idx * inv) >> 21);
+    const Word bit = FG_AT(R.rec(wl), idx - s * row, NRC).bit;
+    return (s << 8) | (bit ? popcw((Word)(bit - 1)) : n2);
+}
+
+// Exact selection: the kept PEDs reach past the histogram window (which starts at A).
+// thr >= 0: offset of the K-th PED, with `below` successors below it.
+template <typename Word, int BK, bool FOLD>
+__device__ __noinline__ void select_exact_warp(const KParams &p,
+                                               const WarpRegs<Word, (BK == 8 ? kMaxB : BK)> R,
+                                               const WarpLevel lv, int A, int newL, int thr,
+                                               int below, uint32_t inv)
+{
+    constexpr int NPL = BK == 8 ? kMaxB : BK;
+    const WarpLayout &wl = p.wl;
+    const int lane = threadIdx.x & 31, row = 4 * lv.nq;
+    const int B = BK == 0 ? 0 : (BK == 2 ? 2 : p.lay.B);
+    int32_t *hist = R.hist(wl);
+    unsigned long long key = 0;
+    int code = 0;
+    int anchor = A;
+    auto score_at = [&](int sh) {
+        for (int b = lane; b < kBuckets; b += 32) FG_AT(hist, b, kBuckets) = 0;
+        __syncwarp();
+        eval_level<Word, BK, FOLD, 1>(p, R, lv, anchor, sh, key, code);
+    };
+    if (thr < 0) {
+        // windows 64 times as wide as the one before until one holds the K-th PED (PEDs are
+        // below 2^16 here), then 64 buckets of 1/64 the width inside the bucket found
+        int sh = 0, pre = 0, first;
+        bool down = false;
+        for (int pass = 0; pass < 12 && !(down && sh == 0); ++pass) {
+            sh += down ? -6 : 6;
+            score_at(sh);
+            find_threshold(p, hist, newL - pre, thr, below, first);
+            __syncwarp();
+            if (thr < kScoreMax) {
+                down = true;
+                pre += below;
+                anchor += thr << sh;
+            }
+        }
+        below = pre;
+    } else {
+        anchor += thr;
     }
-    return lo;
+    score_at(-1);
+    uint32_t *klist = R.klist(wl);
+    compact_bytes(p, R.score(wl), NSC, 0, lv.L * row, 1, newL - below, 0, 0, newL,
+                  [&](int at, int idx, int) { FG_AT(klist, at, FG_N(uint32_t, wl.size[WR_KLIST])) = (uint32_t)idx; });
+    __syncwarp();
+    // PED of every kept child, from the definition; selped holds it in enumeration order
+    for (int x = lane; x < newL; x += 32) {
+        const int cc = warp_code<Word, NPL>(p, R, (int)FG_AT(klist, x, FG_N(uint32_t, wl.size[WR_KLIST])), row, inv, lv.n2);
+        const int s = cc >> 8, j = cc & 0xff;
+        const TgtRec<Word, NPL> t = FG_AT(R.tgt(wl), j, (int64_t)wl.size[WR_TGT] / (int64_t)sizeof(TgtRec<Word, NPL>));
+        Word P = (Word)0, z = (Word)0;
+        int dcnt = 0;
+        for (int q = 0; q < lv.deg; ++q) {
+            const int e = FG_AT(R.nbr(wl), lv.n0 + q, FG_N(int32_t, wl.size[WR_NBR]));
+            const uint8_t ph = FG_AT(R.mapc(wl), (int64_t)s * lv.mrow + (e & 0xffff), wl.size[WR_MAP0]);
+            if (ph == 0xff) { ++dcnt; continue; }
+            const Word pb = (Word)1 << ph;
+            P |= pb;
+            for (int b = 0; b < B; ++b)
+                z |= (((e >> (16 + b)) & 1 ? pb : (Word)0) ^ rec_plane(t, b)) & pb;
+        }
+        const Word im = FG_AT(R.imgc(wl), s, FG_N(Word, wl.size[WR_IMG0])), ai = t.a2 & im;
+        const int crow = FG_AT(R.rec(wl), (int)FG_AT(klist, x, FG_N(uint32_t, wl.size[WR_KLIST])) - s * row, NRC).crow;
+        FG_AT(klist, x, FG_N(uint32_t, wl.size[WR_KLIST])) = (uint32_t)cc;
+        FG_AT(R.selped(wl), x, FG_N(int32_t, wl.size[WR_SELPED])) =
+            FG_AT(R.pedc(wl), s, FG_N(int32_t, wl.size[WR_PED0])) + p.cost.edel * dcnt + crow +
+            p.cost.eins * popcw((Word)(ai & ~P)) + p.cost.edel * popcw((Word)(P & ~t.a2)) +
+            p.cost.esub * popcw((Word)(t.a2 & z));
+    }
+    __syncwarp();
+    // rank by (PED, enumeration order); at most kWarpChunks children per lane
+    int rk[kWarpChunks], pd[kWarpChunks];
+#pragma unroll
+    for (int ch = 0; ch < kWarpChunks; ++ch) {
+        const int x = 32 * ch + lane;
+        rk[ch] = 0;
+        pd[ch] = x < newL ? FG_AT(R.selped(wl), x, FG_N(int32_t, wl.size[WR_SELPED])) : 0;
+        for (int y = 0; x < newL && y < newL; ++y) {
+            const int py = FG_AT(R.selped(wl), y, FG_N(int32_t, wl.size[WR_SELPED]));
+            rk[ch] += py < pd[ch] || (py == pd[ch] && y < x);
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int ch = 0; ch < kWarpChunks; ++ch) {
+        const int x = 32 * ch + lane;
+        if (x < newL) {
+            FG_AT(R.sel(wl), rk[ch], FG_N(int32_t, wl.size[WR_SEL])) = (int)FG_AT(klist, x, FG_N(uint32_t, wl.size[WR_KLIST]));
+            FG_AT(R.selped(wl), rk[ch], FG_N(int32_t, wl.size[WR_SELPED])) = pd[ch];
+        }
+    }
+    __syncwarp();
 }
 
 template <typename Word, int BK, bool FOLD>
@@ -397,28 +448,26 @@ __device__ __forceinline__ void solve_pair_warp(const KParams &p, uint32_t wb, u
     const int B = BK == 0 ? 0 : (BK == 2 ? 2 : p.lay.B);
     const int mrow = wl.mrow;
     const CostModel c = p.cost;
-    // buckets 0..H-2 hold one PED offset each; a K-th offset past them takes the exact fallback
-    const int H = min(p.hwin, kWarpBuckets);
+    const int hwin = p.hwin;   // PEDs a kept list may span without the exact selection
     constexpr uint8_t DEL = 0xff;
     // m &= ballot(bit b of an offset) ^ lb[b] keeps the lanes whose bit b equals bit b of
     // this lane's index
-    unsigned lb[4];
+    unsigned lb[5];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) lb[k] = ((lane >> k) & 1) ? 0u : 0xffffffffu;
+    for (int k = 0; k < 5; ++k) lb[k] = ((lane >> k) & 1) ? 0u : 0xffffffffu;
 #ifdef FASTGED_PHASE_TIMERS
     long long ph[16] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     long long ph_last = clock64();
 #endif
 
-    // ---- stage the target graph (record u + 1 target vertex u, record n2 + 1 the deletion,
-    // record 0 the stand-in of finished walks) and the source graph's prior-neighbour lists
+    // ---- stage the target graph (record u target vertex u, record n2 the deletion) and the
+    // source graph's prior-neighbour lists
     {
         const uint64_t *adj2 = p.adj + m2.adj_off;
         const uint64_t *pl2 = p.planes + m2.plane_off;
         const int W2 = m2.W;
-        for (int k = lane; k <= n2 + 1; k += 32) {
-            const int u = k - 1;
-            const bool vtx = u >= 0 && u < n2;
+        for (int u = lane; u <= n2; u += 32) {
+            const bool vtx = u < n2;
             Rec r;
             r.a2 = vtx ? (Word)FG_AT(adj2, (int64_t)u * W2, p.adj_words - m2.adj_off) : (Word)0;
 #pragma unroll
@@ -427,8 +476,8 @@ __device__ __forceinline__ void solve_pair_warp(const KParams &p, uint32_t wb, u
                                         ? (Word)FG_AT(pl2, ((int64_t)b * n2 + u) * W2,
                                                       p.plane_words - m2.plane_off)
                                         : (Word)0);
-            r.crow = k == 0 ? kWarpIdleCost : 0;
-            FG_AT(R.tgt(wl), k, WN(Rec, WR_TGT)) = r;
+            r.crow = 0;
+            FG_AT(R.tgt(wl), u, WN(Rec, WR_TGT)) = r;
             if (vtx)
                 FG_AT(R.lab2(wl), u, WN(int32_t, WR_LAB2)) =
                     FG_AT(p.vlab, m2.lab_off + u, p.n_vlab);
@@ -487,95 +536,133 @@ __device__ __forceinline__ void solve_pair_warp(const KParams &p, uint32_t wb, u
 
     long long nevals = 0;
     int L = 1;
+    Word all = (Word)0;   // target vertices that every node uses
+    const Word nmask = n2 >= WB ? ~(Word)0 : (((Word)1 << n2) - (Word)1);
+    using CRec = WarpRec<Word>;
     WPHASE(0);
     for (int i = 0; i < n1; ++i) {
-        // S1: this level's vertex-cost row C[i][u] in quarter units (record n2 + 1, the
-        // deletion column, holds c_vdel; record 0 keeps its stand-in cost)
+        // the level's active columns, increasing: vertices not used by every node, and the
+        // deletion as bit n2 (n2 < WB); their records with S1, the vertex-cost row C[i][.], and
+        // one-hot vertex bits; past them, up to an odd number of quads (the lanes' rows then
+        // fall into different banks), columns that score past every bucket
+        const Word actm = (Word)((~all & nmask) | ((Word)1 << n2));
+        const int nact = popcw(actm), nq = (nact + 3) / 4 | 1;
+        WarpLevel lv;
+        lv.L = L;
+        lv.n0 = FG_AT(R.noff(wl), i, WN(int32_t, WR_NOFF));
+        lv.deg = FG_AT(R.noff(wl), i + 1, WN(int32_t, WR_NOFF)) - lv.n0;
+        lv.n2 = n2;
+        lv.mrow = mrow;
+        lv.nq = nq;
+        lv.nk = (nact + 3) / 4;
+        lv.m2 = m2.m;
+        // the label of v_i's edges to its prior neighbours, when they have one
+        int lab = 0;
+        lv.one_label = true;
+        if (NPL > 0 && lv.deg > 0) {
+            lab = FG_AT(R.nbr(wl), lv.n0, WN(int32_t, WR_NBR)) >> 16;
+            for (int t = 1; t < lv.deg; ++t)
+                lv.one_label &= (FG_AT(R.nbr(wl), lv.n0 + t, WN(int32_t, WR_NBR)) >> 16) == lab;
+        }
         {
             const int a1 = FG_AT(p.vlab, m1.lab_off + i, p.n_vlab);
-            for (int k = lane + 1; k <= n2 + 1; k += 32)
-                FG_AT(R.tgt(wl), k, WN(Rec, WR_TGT)).crow =
-                    4 * (k <= n2 ? ((FG_AT(R.lab2(wl), k - 1, WN(int32_t, WR_LAB2)) != a1) ? c.vsub : 0)
-                                 : c.vdel);
+            for (int u = lane; u <= n2; u += 32) {
+                if (!((actm >> u) & (Word)1)) continue;
+                const int pos = popcw((Word)(actm & (((Word)1 << u) - (Word)1)));
+                const Rec t = FG_AT(R.tgt(wl), u, WN(Rec, WR_TGT));
+                CRec cr;
+                cr.a2 = t.a2;
+                Word ld = (Word)0;
+#pragma unroll
+                for (int b = 0; b < NPL; ++b) {
+                    ld |= rec_plane(t, b) ^ ((lab >> b) & 1 ? ~(Word)0 : (Word)0);
+                    if (!lv.one_label && b < B) FG_AT(R.planes(wl), b * 4 * nq + pos, NPA) = rec_plane(t, b);
+                }
+                cr.mis = t.a2 & ld;
+                cr.bit = u < n2 ? (Word)1 << u : (Word)0;
+                cr.crow = u < n2 ? ((FG_AT(R.lab2(wl), u, WN(int32_t, WR_LAB2)) != a1) ? c.vsub : 0) : c.vdel;
+                FG_AT(R.rec(wl), pos, NRC) = cr;
+            }
+            if (lane < 4 * nq - nact) {   // fewer than eight
+                CRec cr = {};
+                cr.crow = kWarpPadCost;
+                FG_AT(R.rec(wl), nact + lane, NRC) = cr;
+                if (!lv.one_label)
+                    for (int b = 0; b < B; ++b) FG_AT(R.planes(wl), b * 4 * nq + nact + lane, NPA) = (Word)0;
+            }
+            for (int b = lane; b < kBuckets; b += 32) FG_AT(R.hist(wl), b, kBuckets) = 0;
         }
         __syncwarp();
         WPHASE(7);
-        const int n0 = FG_AT(R.noff(wl), i, WN(int32_t, WR_NOFF));
-        const int deg = FG_AT(R.noff(wl), i + 1, WN(int32_t, WR_NOFF)) - n0;
         const int A = FG_AT(R.pedc(wl), 0, WN(int32_t, WR_PED0));   // least PED of the kept list: a lower bound of every child
-        int hist = 0;
+        unsigned long long key = ~0ull;
+        int code = INT_MAX;
+        if (p.variant == 1 && i == n1 - 1) {
+            // variant B: every successor of the last level is completed, and the least (total,
+            // PED, enumeration order) wins
+            const int tot = eval_level<Word, BK, FOLD, 2>(p, R, lv, A, 0, key, code);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long k2 = __shfl_xor_sync(FULL, key, o);
+                const int c2 = __shfl_xor_sync(FULL, code, o);
+                if (k2 < key || (k2 == key && c2 < code)) {
+                    key = k2;
+                    code = c2;
+                }
+            }
+            if (lane == 0) {
+                FG_AT(p.out_cost, pair, p.n_pairs) = (int32_t)(key >> 32);
+                if (p.out_nevals) FG_AT(p.out_nevals, pair, p.n_pairs) = nevals + 2LL * tot;
+            }
+            const int64_t mo = FG_AT(p.map_off, pair, p.n_pairs);
+            const int ws = code >> 8, wj = code & 0xff;
+            for (int k = lane; k < n1; k += 32) {
+                const uint8_t v = k == i ? (wj < n2 ? (uint8_t)wj : DEL)
+                                         : FG_AT(R.mapc(wl), (int64_t)ws * mrow + k, wl.size[WR_MAP0]);
+                FG_AT(p.out_map, mo + k, p.map_total) = v == DEL ? -1 : (int32_t)v;
+            }
+            __syncwarp();
+            return;
+        }
 #ifdef FASTGED_PHASE_TIMERS
-        const int tot = eval_level<Word, BK, FOLD, false>(p, R, L, n0, deg, n2, mrow, A, hist,
-                                                          ph);
-        ph[10] += tot;   // successors (the loop steps above cover them 32 lanes at a time)
+        const int tot = eval_level<Word, BK, FOLD, 0>(p, R, lv, A, 0, key, code, ph);
+        ph[10] += tot;   // successors
         ph[11] += 1;     // levels
 #else
-        const int tot = eval_level<Word, BK, FOLD, false>(p, R, L, n0, deg, n2, mrow, A, hist);
+        const int tot = eval_level<Word, BK, FOLD, 0>(p, R, lv, A, 0, key, code);
 #endif
         nevals += tot;
         WPHASE(1);
         const int newL = min(K, tot);
-        // S4: bucket b = PED - A for b < H - 1; a K-th offset past them goes to the exact
-        // fallback
-        const int cb = lane < H - 1 ? hist : 0;
-        int incl = cb;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(FULL, incl, o);
-            if (lane >= o) incl += v;
-        }
-        const int bexcl = incl - cb;
-        const unsigned hb = __ballot_sync(FULL, lane < H - 1 && incl >= newL);
-        if (hb) {
-            const int thr = __ffs(hb) - 1;
+        const int row = 4 * nq;
+        const uint32_t inv = ((1u << 21) + (uint32_t)row - 1u) / (uint32_t)row;
+        // S4: bucket b = PED - A; kept PEDs past the window or over too many buckets go to the
+        // exact selection
+        int thr, below, first;
+        find_threshold(p, R.hist(wl), newL, thr, below, first);
+        if (thr < kScoreMax && thr - first < hwin - 1) {
             // kept: every successor below bucket thr and the first q of bucket thr, compacted
-            // in enumeration order (the loop stops once all are found)
-            const int q = newL - __shfl_sync(FULL, bexcl, thr);
-            const int lim = (thr + 1) << 8;   // entry < lim <=> PED offset <= thr
-            int keep_before = 0, eq_before = 0;
-            for (int kb = 0; kb < tot && keep_before < newL; kb += 128) {
-                int e[4];
-                unsigned le[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int k = kb + 32 * u + lane;
-                    e[u] = k < tot ? (int)FG_AT(R.ent(wl), k, WN(uint16_t, WR_ENT)) : 0xffff;
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) le[u] = __ballot_sync(FULL, e[u] < lim);
-                if ((le[0] | le[1] | le[2] | le[3]) == 0u) continue;
-                // the four sub-chunks' ties, then their kept sets, each set of ballots taken
-                // together (the counts of the sub-chunks before are prefix sums)
-                const unsigned lt = lanemask_lt();
-                unsigned eqb[4], kbm[4];
-                bool keep[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) eqb[u] = __ballot_sync(FULL, (e[u] >> 8) == thr);
-                int eqp = eq_before;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int d = e[u] >> 8;
-                    keep[u] = (d < thr) || (d == thr && eqp + __popc(eqb[u] & lt) < q);
-                    eqp += __popc(eqb[u]);
-                }
-                eq_before = eqp;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) kbm[u] = __ballot_sync(FULL, keep[u]);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (keep[u])
-                        FG_AT(R.klist(wl), keep_before + __popc(kbm[u] & lt), WN(uint32_t, WR_KLIST)) =
-                            ((uint32_t)e[u] << 16) | (uint32_t)(kb + 32 * u + lane);
-                    keep_before += __popc(kbm[u]);
-                }
-            }
+            // in enumeration order (score byte << 16 | its index; at most 128 * 72 bytes)
+            const int q = newL - below;
+            uint32_t *klist = R.klist(wl);
+            compact_bytes(p, R.score(wl), NSC, 0, L * row, thr, q, 0, 0, newL,
+                          [&](int at, int idx, int v) {
+                              FG_AT(klist, at, WN(uint32_t, WR_KLIST)) = ((uint32_t)(v - first) << 16) | (uint32_t)idx;
+                          });
             __syncwarp();
             WPHASE(3);
             // place every kept successor at its rank: (smaller offsets) + (equal offsets
             // earlier in enumeration order). All chunks of the kept list are handled at once;
-            // lane b carries the kept successors of bucket b in the chunks before each one.
-            // A kept entry is its 16-bit successor entry (offset << 8 | record index) << 16 |
-            // its index k in enumeration order.
+            // lane b carries the kept successors of bucket first + b in the chunks before each
+            // one.
+            int incl = first + lane < thr ? FG_AT(R.hist(wl), first + lane, kBuckets) : 0;
+            const int cb = incl;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const int bexcl = incl - cb;
             uint32_t kv[kWarpChunks];
             int dk[kWarpChunks], pos[kWarpChunks];
             bool vk[kWarpChunks];
@@ -585,16 +672,18 @@ __device__ __forceinline__ void solve_pair_warp(const KParams &p, uint32_t wb, u
                 const int x = 32 * ch + lane;
                 vk[ch] = x < newL;
                 kv[ch] = vk[ch] ? FG_AT(R.klist(wl), x, WN(uint32_t, WR_KLIST)) : 0u;
-                dk[ch] = (int)(kv[ch] >> 24);
+                dk[ch] = (int)(kv[ch] >> 16);
             }
 #pragma unroll
             for (int ch = 0; ch < kWarpChunks; ++ch) {
+                if (32 * ch >= newL) break;
                 const unsigned V = __ballot_sync(FULL, vk[ch]);
                 // same: lanes whose offset equals this lane's; m: lanes whose offset is this
                 // lane's index
                 unsigned same = V, m = V;
 #pragma unroll
-                for (int b = 0; b < 4; ++b) {
+                for (int b = 0; b < 5; ++b) {
+                    if ((thr - first) >> b == 0) break;   // no offset has this bit
                     const unsigned bb = __ballot_sync(FULL, (dk[ch] >> b) & 1);
                     same &= ((dk[ch] >> b) & 1) ? bb : ~bb;
                     m &= bb ^ lb[b];
@@ -603,94 +692,17 @@ __device__ __forceinline__ void solve_pair_warp(const KParams &p, uint32_t wb, u
                           __popc(same & lanemask_lt());
                 run += __popc(m);
             }
-            // parent slot of every kept entry: the last node whose first entry is at or
-            // before it, by a branch-free binary search over nodeoff (L <= kWarpChunks * 32),
-            // the chunks' searches interleaved so that their loads overlap
-            int sl[kWarpChunks];
-#pragma unroll
-            for (int ch = 0; ch < kWarpChunks; ++ch) sl[ch] = 0;
-            for (int st = L > 1 ? 1 << (31 - __clz(L - 1)) : 0; st > 0; st >>= 1) {
-#pragma unroll
-                for (int ch = 0; ch < kWarpChunks; ++ch) {
-                    const int m = sl[ch] + st;
-                    if (m < L && (int)FG_AT(R.nodeoff(wl), m, WN(uint16_t, WR_NODEOFF)) <=
-                                     (int)(kv[ch] & 0xffffu))
-                        sl[ch] = m;
-                }
-            }
 #pragma unroll
             for (int ch = 0; ch < kWarpChunks; ++ch) {
                 if (vk[ch]) {
                     FG_AT(R.sel(wl), pos[ch], WN(int32_t, WR_SEL)) =
-                        (sl[ch] << 8) | (int)((kv[ch] >> 16) & 0xffu);
-                    FG_AT(R.selped(wl), pos[ch], WN(int32_t, WR_SELPED)) = A + dk[ch];
+                        warp_code<Word, NPL>(p, R, (int)(kv[ch] & 0xffffu), row, inv, n2);
+                    FG_AT(R.selped(wl), pos[ch], WN(int32_t, WR_SELPED)) = A + first + dk[ch];
                 }
             }
             WPHASE(4);
         } else {
-            // exact fallback: score the level again with exact PED offsets, find the K-th one
-            // by bisection, compact the kept entries in enumeration order and rank them by
-            // (PED, enumeration order)
-            int dummy = 0;
-            eval_level<Word, BK, FOLD, true>(p, R, L, n0, deg, n2, mrow, A, dummy);
-            auto count_le = [&](int t) -> int {
-                int cnt = 0;
-                for (int k = lane; k < tot; k += 32)
-                    cnt += ((int)FG_AT(R.ent(wl), k, WN(uint16_t, WR_ENT)) <= t);
-                return warp_sum(cnt);
-            };
-            int lo = H - 1, hi = 0;
-            for (int k = lane; k < tot; k += 32)
-                hi = max(hi, (int)FG_AT(R.ent(wl), k, WN(uint16_t, WR_ENT)));
-            hi = (int)__reduce_max_sync(FULL, (unsigned)hi);
-            if (lo > hi) lo = hi;
-            while (lo < hi) {   // count(<= lo - 1) < newL <= count(<= hi)
-                const int mid = lo + (hi - lo) / 2;
-                if (count_le(mid) >= newL) hi = mid;
-                else lo = mid + 1;
-            }
-            const int T = lo;
-            const int q = newL - (T > 0 ? count_le(T - 1) : 0);
-            int keep_before = 0, eq_before = 0;
-            for (int kb = 0; kb < tot; kb += 32) {
-                const int k = kb + lane;
-                const int d = k < tot ? (int)FG_AT(R.ent(wl), k, WN(uint16_t, WR_ENT)) : 0x10000;
-                const bool is_eq = d == T;
-                const unsigned eqb = __ballot_sync(FULL, is_eq);
-                const bool keep = (d < T) || (is_eq && eq_before + __popc(eqb & lanemask_lt()) < q);
-                const unsigned kbm = __ballot_sync(FULL, keep);
-                if (keep)
-                    FG_AT(R.klist(wl), keep_before + __popc(kbm & lanemask_lt()), WN(uint32_t, WR_KLIST)) =
-                        ((uint32_t)d << 16) | (uint32_t)k;
-                keep_before += __popc(kbm);
-                eq_before += __popc(eqb);
-            }
-            __syncwarp();
-            // rank of every kept key (keys are distinct: the entry index is in the low half)
-            for (int x = lane; x < newL; x += 32) {
-                const uint32_t kx = FG_AT(R.klist(wl), x, WN(uint32_t, WR_KLIST));
-                int rank = 0;
-                for (int y = 0; y < newL; ++y) rank += FG_AT(R.klist(wl), y, WN(uint32_t, WR_KLIST)) < kx;
-                FG_AT(R.selped(wl), rank, WN(int32_t, WR_SELPED)) = (int)kx;
-            }
-            __syncwarp();
-            for (int r = lane; r < newL; r += 32) {
-                const uint32_t kx = (uint32_t)FG_AT(R.selped(wl), r, WN(int32_t, WR_SELPED));
-                const int d = (int)(kx >> 16), k = (int)(kx & 0xffffu);
-                const int s = node_of(p, R.nodeoff(wl), L, k);
-                const int no = (int)FG_AT(R.nodeoff(wl), s, WN(uint16_t, WR_NODEOFF));
-                const int t = k - no;
-                const int cnt = (int)FG_AT(R.nodeoff(wl), s + 1, WN(uint16_t, WR_NODEOFF)) - no;
-                int j = n2 + 1;      // record index: the deletion
-                if (t < cnt - 1) {   // the t-th free target vertex of node s
-                    const Word nmask = n2 >= WB ? ~(Word)0 : (((Word)1 << n2) - (Word)1);
-                    Word x = ~FG_AT(R.imgc(wl), s, WN(Word, WR_IMG0)) & nmask;
-                    for (int z = 0; z < t; ++z) x &= x - (Word)1;
-                    j = ffs1(x);
-                }
-                FG_AT(R.sel(wl), r, WN(int32_t, WR_SEL)) = (s << 8) | j;
-                FG_AT(R.selped(wl), r, WN(int32_t, WR_SELPED)) = A + d;
-            }
+            select_exact_warp<Word, BK, FOLD>(p, R, lv, A, newL, thr < kScoreMax ? thr : -1, below, inv);
             WPHASE(5);
         }
         __syncwarp();
@@ -700,9 +712,10 @@ __device__ __forceinline__ void solve_pair_warp(const KParams &p, uint32_t wb, u
             const int nvec = (i + 15) >> 4;
             const uint8_t *__restrict__ mapc = R.mapc(wl);
             uint8_t *__restrict__ mapn = R.mapn(wl);
+            Word am = ~(Word)0;
             for (int r = lane; r < newL; r += 32) {
                 const int v = FG_AT(R.sel(wl), r, WN(int32_t, WR_SEL));
-                const int s = v >> 8, jr = v & 0xff, j = jr - 1;   // record index, vertex (n2: deletion)
+                const int s = v >> 8, j = v & 0xff;   // parent, vertex (n2: deletion)
                 const int64_t src = (int64_t)s * (mrow >> 4), dst = (int64_t)r * (mrow >> 4);
                 for (int t = 0; t < nvec; ++t)
                     FG_AT((uint4 *)mapn, dst + t, FG_N(uint4, wl.size[WR_MAP0])) =
@@ -712,13 +725,17 @@ __device__ __forceinline__ void solve_pair_warp(const KParams &p, uint32_t wb, u
                 int e2 = FG_AT(R.e2c(wl), s, WN(uint16_t, WR_E20));
                 Word imn = im;
                 if (j < n2) {
-                    e2 += popcw((Word)(FG_AT(R.tgt(wl), jr, WN(Rec, WR_TGT)).a2 & im));
+                    e2 += popcw((Word)(FG_AT(R.tgt(wl), j, WN(Rec, WR_TGT)).a2 & im));
                     imn |= (Word)1 << j;
                 }
                 FG_AT(R.imgn(wl), r, WN(Word, WR_IMG0)) = imn;
+                am &= imn;
                 FG_AT(R.e2n(wl), r, WN(uint16_t, WR_E20)) = (uint16_t)e2;
                 FG_AT(R.pedn(wl), r, WN(int32_t, WR_PED0)) = FG_AT(R.selped(wl), r, WN(int32_t, WR_SELPED));
             }
+            all = (Word)__reduce_and_sync(FULL, (unsigned)am);
+            if (WB == 64)
+                all |= (Word)((uint64_t)__reduce_and_sync(FULL, (unsigned)((uint64_t)am >> 32)) << 32);
         }
         __syncwarp();
         R.cur ^= 1;
@@ -759,6 +776,9 @@ __device__ __forceinline__ void solve_pair_warp(const KParams &p, uint32_t wb, u
         for (int k = 0; k < 16; ++k) atomicAdd(&p.phase_cycles[k], (unsigned long long)ph[k]);
 #endif
 #undef WN
+#undef NSC
+#undef NRC
+#undef NPA
 }
 
 // Persistent one-warp teams: each warp pops pairs from the class's queue until it is empty.

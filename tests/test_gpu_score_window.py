@@ -55,3 +55,32 @@ def test_anchor_jumps(cluster, clique_first, scale):
     g1 = _clique_and_isolated(36, clique_first)
     w = single([(g1, W.erdos_renyi(st, 140, 0.3, 3)), (g1, W.erdos_renyi(st, 30, 0.6, 3))], costs, 30)
     assert_parity(w, gpu_run(w, team=F.FASTGED_TEAM_CTA, cluster=cluster))
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("n2", [1, 2, 3, 4, 7, 8, 15, 16, 30, 31, 32, 33, 62, 63])
+def test_one_warp_column_edges(n2, variant):
+    st = W.Stream(n2, 8)
+    w = single([(_labelled(st, n1, 0.4), _labelled(st, n2, 0.3)) for n1 in (1, 9, 31)],
+               W.SETTING1_COSTS, 40)
+    assert_parity(w, gpu_run(w, variant=variant), variant=variant)
+
+
+@pytest.mark.parametrize("K", [1, 2, 3, 5, 9, 17, 31, 33, 97, 127, 128])
+def test_one_warp_beam_edges(K):
+    st = W.Stream(K, 9)
+    w = single([(_labelled(st, 12, 0.3), _labelled(st, n, 0.3)) for n in (8, 20, 40)],
+               W.SETTING2_COSTS, K)
+    for window in (0, 2, 17):
+        assert_parity(w, gpu_run(w, hist_window=window))
+
+
+@pytest.mark.parametrize("scale", [1, 9, 120])
+def test_one_warp_wide_offsets(scale):
+    """PED offsets past the 127 of a score byte, up to the 16 bits a one-warp pair allows."""
+    costs = tuple(scale * c for c in W.SETTING1_COSTS)
+    st = W.Stream(scale, 10)
+    w = single([(_clique_and_isolated(16, f), W.erdos_renyi(st, 25, 0.5, 3)) for f in (False, True)],
+               costs, 60)
+    for variant in (0, 1):
+        assert_parity(w, gpu_run(w, variant=variant), variant=variant)
