@@ -412,14 +412,35 @@ __device__ __forceinline__ void score_table(const KParams &p, const Regions<Word
     const uint8_t *a2b = (const uint8_t *)R.a2t, *imb = (const uint8_t *)V.imgw;
     const int64_t NA = p.lay.rsize[RG_A2T], NE = p.lay.rsize[RG_ET0];
     constexpr int WBY = (int)sizeof(Word);
+    // the parents' rows come from L2 or DRAM (all teams' rows: 150 MB on 64 large pairs), so a
+    // whole row of the next node is under way while a node is scored
+    constexpr int KS = (64 * W + 8 + 255) / 256;   // steps of a row at most
+    uint2 nxt[KS];
+    auto fetch = [&](int t) {
+        const int par = __shfl_sync(0xffffffffu, nd.code, t) >> kSelShift;
+#pragma unroll
+        for (int k = 0; k < KS; ++k) {
+            const int c0 = 256 * k + 8 * lane;
+            nxt[k] = make_uint2(0u, 0u);
+            if (!root && c0 < V.stride) nxt[k] = FG_AT((const uint2 *)ec, ((int64_t)par * N2S + c0) >> 3, NE >> 3);
+        }
+    };
+    fetch(0);
     for (int t = 0; t < ng; ++t) {
         const int s = g0 + t;
+        uint2 cur[KS];
+#pragma unroll
+        for (int k = 0; k < KS; ++k) cur[k] = nxt[k];
+        if (t + 1 < ng) fetch(t + 1);
         const int code = __shfl_sync(0xffffffffu, nd.code, t);
         const int np = __shfl_sync(0xffffffffu, nd.nimg, t);
         const int base = __shfl_sync(0xffffffffu, nd.base, t) + (FOLD ? 0 : c_edel * np);
         const uint32_t p0 = __shfl_sync(0xffffffffu, nd.ph[0], t), p1 = __shfl_sync(0xffffffffu, nd.ph[1], t);
-        const int par = code >> kSelShift, jc = code & ((1 << kSelShift) - 1);
-        for (int c0 = 8 * lane; c0 < V.stride; c0 += 256) {
+        const int jc = code & ((1 << kSelShift) - 1);
+#pragma unroll
+        for (int k = 0; k < KS; ++k) {
+            const int c0 = 256 * k + 8 * lane;
+            if (c0 >= V.stride) break;
             const int wrow = (c0 / (8 * WBY)) * N2S, by = (c0 >> 3) % WBY;   // word row, byte in it
             // bits c0 .. c0 + 7 of row u of A2 (columns and rows of A2 are alike; row n2 is empty)
             // (columns past the last word: none)
@@ -429,10 +450,9 @@ __device__ __forceinline__ void score_table(const KParams &p, const Regions<Word
             };
             uint32_t e[2] = {0u, 0u};
             if (!root) {
-                const uint2 x = FG_AT((const uint2 *)ec, ((int64_t)par * N2S + c0) >> 3, NE >> 3);
                 const uint32_t a = bits(jc);
-                e[0] = x.x + nibble_bytes(a);
-                e[1] = x.y + nibble_bytes(a >> 4);
+                e[0] = cur[k].x + nibble_bytes(a);
+                e[1] = cur[k].y + nibble_bytes(a >> 4);
             }
             FG_AT((uint2 *)en, ((int64_t)s * N2S + c0) >> 3, NE >> 3) = make_uint2(e[0], e[1]);
             uint32_t tt[2] = {0u, 0u};
@@ -447,8 +467,8 @@ __device__ __forceinline__ void score_table(const KParams &p, const Regions<Word
             if (deg > 2) image(p1 & 0xffffu);
             if (deg > 3) image(p1 >> 16);
             for (int q = 4; q < deg; ++q) {
-                const int k = FG_AT(R.nbr, n0 + q, FG_N(int32_t, p.lay.rsize[RG_NBR])) & 0xffff;
-                image((uint32_t)FG_AT(map, (int64_t)s * mt + k, FG_N(MapT, p.lay.rsize[RG_MAP0])));
+                const int v = FG_AT(R.nbr, n0 + q, FG_N(int32_t, p.lay.rsize[RG_NBR])) & 0xffff;
+                image((uint32_t)FG_AT(map, (int64_t)s * mt + v, FG_N(MapT, p.lay.rsize[RG_MAP0])));
             }
             // used columns and the ones past the deletion
             uint32_t um = c0 < n2 ? (uint32_t)FG_AT(imb, (int64_t)(s - V.ioff) * W * WBY + (c0 >> 3), V.nimg * WBY) : 0u;
@@ -1379,21 +1399,53 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
                     }
                 }
             } else {
-                // cluster teams: a warp per child
-                for (int r = warp; r < newL; r += NW) {
-                    const int v = FG_AT(R.sel, r, FG_N(int32_t, p.lay.rsize[RG_SEL]));
-                    const int s = v >> kSelShift, j = v & ((1 << kSelShift) - 1);
-                    for (int t = lane; t < nvec; t += 32)
-                        FG_AT((uint4 *)mapn, r * m16 + t, NMAP16) = FG_AT((const uint4 *)mapc, s * m16 + t, NMAP16);
-                    for (int w = lane; w < W; w += 32) {
-                        Word x = FG_AT(imgc, (int64_t)s * W + w, NIMG);
-                        if (j < n2 && j / WB == w) x |= (Word)1 << (j % WB);
-                        FG_AT(imgn, (int64_t)r * W + w, NIMG) = x;
-                    }
-                    __syncwarp();
-                    if (lane == 0) {
-                        FG_AT((MapT *)mapn, r * mt + i, NMAPT) = (j < n2) ? (MapT)j : DEL;
-                        FG_AT(pedn, r, NPED) = FG_AT(R.selped, r, FG_N(int32_t, p.lay.rsize[RG_SELPED]));
+                // cluster teams: a warp copies its children two at a time. Its next 32 codes and
+                // PEDs come in one load each, and up to four map vectors per lane are under way
+                // (rows of up to 2 KB from L2: with one vector under way the copies took a
+                // fifth of the time on large pairs)
+                for (int rb = warp; rb < newL; rb += 32 * NW) {
+                    const int mine = rb + lane * NW;
+                    const int mc = mine < newL ? FG_AT(R.sel, mine, FG_N(int32_t, p.lay.rsize[RG_SEL])) : 0;
+                    const int md = mine < newL ? FG_AT(R.selped, mine, FG_N(int32_t, p.lay.rsize[RG_SELPED])) : 0;
+                    const int cnt = min(32, (newL - rb + NW - 1) / NW);
+                    for (int t = 0; t < cnt; t += 2) {
+                        const int ca = __shfl_sync(0xffffffffu, mc, t), cb = __shfl_sync(0xffffffffu, mc, (t + 1) & 31);
+                        const int da = __shfl_sync(0xffffffffu, md, t), db = __shfl_sync(0xffffffffu, md, (t + 1) & 31);
+                        const bool two = t + 1 < cnt;
+                        const int64_t ra = rb + (int64_t)t * NW, rc = two ? ra + NW : ra;
+                        const int64_t sa = ca >> kSelShift, sb = (two ? cb : ca) >> kSelShift;
+                        for (int v = lane; v < nvec; v += 64) {
+                            const bool w2 = v + 32 < nvec;
+                            uint4 x[4];
+                            x[0] = FG_AT((const uint4 *)mapc, sa * m16 + v, NMAP16);
+                            x[1] = FG_AT((const uint4 *)mapc, sb * m16 + v, NMAP16);
+                            if (w2) {
+                                x[2] = FG_AT((const uint4 *)mapc, sa * m16 + v + 32, NMAP16);
+                                x[3] = FG_AT((const uint4 *)mapc, sb * m16 + v + 32, NMAP16);
+                            }
+                            FG_AT((uint4 *)mapn, ra * m16 + v, NMAP16) = x[0];
+                            if (two) FG_AT((uint4 *)mapn, rc * m16 + v, NMAP16) = x[1];
+                            if (w2) {
+                                FG_AT((uint4 *)mapn, ra * m16 + v + 32, NMAP16) = x[2];
+                                if (two) FG_AT((uint4 *)mapn, rc * m16 + v + 32, NMAP16) = x[3];
+                            }
+                        }
+                        __syncwarp();
+                        // half a warp per child: Img words (16 at most), entry i, PED
+                        const bool hi = lane >= 16;
+                        if (!hi || two) {
+                            const int j = (hi ? cb : ca) & ((1 << kSelShift) - 1), w = lane & 15;
+                            const int64_t r = hi ? rc : ra, s = hi ? sb : sa;
+                            if (w < W) {
+                                Word x = FG_AT(imgc, s * W + w, NIMG);
+                                if (j < n2 && j / WB == w) x |= (Word)1 << (j % WB);
+                                FG_AT(imgn, r * W + w, NIMG) = x;
+                            }
+                            if (w == 0) {
+                                FG_AT((MapT *)mapn, r * mt + i, NMAPT) = (j < n2) ? (MapT)j : DEL;
+                                FG_AT(pedn, r, NPED) = hi ? db : da;
+                            }
+                        }
                     }
                 }
             }
