@@ -116,7 +116,8 @@ typedef struct {
                              /* source index order either way                                 */
     int32_t team;            /* FASTGED_TEAM_AUTO (0): pairs with at most 64 vertices in g1,  */
                              /* at most 63 in g2 and K <= 128 are solved by one warp each,    */
-                             /* the others by a CTA (or a cluster of CTAs) each;              */
+                             /* (in batches of few pairs with K >= 64 by a CTA each), the      */
+                             /* others by a CTA (or a cluster of CTAs) each;                  */
                              /* FASTGED_TEAM_CTA (1): every pair by a CTA or cluster.         */
                              /* Results do not depend on it                                   */
     int32_t max_sms;         /* 0 = no cap; else the resident teams of each size class are   */

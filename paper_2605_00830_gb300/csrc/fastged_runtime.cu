@@ -689,6 +689,22 @@ static bool cluster_eligible(const ClassPlan &cp, int npairs, int sm_count)
     return cp.W >= 4 || (int64_t)cp.kmax * (cp.n2max + 1) >= 16384;
 }
 
+// A batch of few pairs leaves most warps of the GPU without one, and takes as long as one warp
+// needs for its largest pair: a CTA per pair is then faster. Measured at K = 100 on pairs of
+// 10-40 vertices, whole calls, one-warp and 256-thread teams: 1 pair 201 and 138 us, 100 pairs
+// 571 and 320, 500 pairs 626 and 412, 1,001 pairs 688 and 597, 2,000 pairs 878 and 952; up to
+// 14 vertices 500 pairs 177 and 202. At K = 16 one warp is the faster one for any number (100
+// pairs: 204 and 263). A class whose one-warp shapes are being timed stays with them (its
+// sample is smaller than the batch it stands for).
+static bool team_beats_warps(const ClassPlan &cp, int n_pairs, int sm_count)
+{
+    {
+        std::lock_guard<std::mutex> g(g_tune_mu);
+        if (g_tune_forcing && g_tune_force.gmap >= 0) return false;
+    }
+    return cp.kmax >= 64 && cp.n1max >= 16 && n_pairs <= 8 * sm_count;
+}
+
 // CTAs per cluster without a tuning entry. A handful of pairs (16 CTAs each still fit the GPU
 // at once) takes 16: measured on 8 and 16 CTAs, one G(200, 0.4) pair 28.4 and 13.5 ms at
 // K = 5,000, 4.9 and 3.9 ms at K = 500; 4 pairs of 20 vertices 10.8 and 5.9 ms at K = 100,000;
@@ -1185,6 +1201,7 @@ int fastged::flatten(fastged_handle *h, const fastged_pair_list *pl, int32_t K,
     }
     b.map_total = mtot;
     for (auto &cp : b.classes) {
+        if (cp.warp && team_beats_warps(cp, np, h->sm_count)) cp.warp = false;
         int rc = tune_class(h, cp, B, opt.block_threads, opt.max_sms, opt.cluster);
         if (rc) return rc;
     }
