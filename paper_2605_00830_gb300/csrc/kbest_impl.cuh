@@ -1033,14 +1033,16 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
             if (lane < W32) atomicAnd(&FG_AT(R.allm, lane, FG_N(uint32_t, p.lay.rsize[RG_ALL])), am);
         }
         __syncthreads();
-        // active columns, increasing: the vertices not used by all, and the deletion n2
-        int nact = n2 + 1, stride;
+        // active columns, increasing: the vertices not used by all, and the deletion n2. None
+        // for a cluster CTA without nodes (levels of fewer nodes than CTAs): its used-by-all mask
+        // is still all ones and its column list is not written, so no pass may read it
+        int nact = cs1 > cs0 ? n2 + 1 : 0, stride;
         {
             using Rec = ColRec<Word, (BK == 8 ? kMaxB : BK)>;
             constexpr int NPL = BK == 8 ? kMaxB : BK;
             Word *jm = (Word *)((uint8_t *)R.rec + p.lay.jm_off);   // one-hot vertex bits
 #define NJM FG_N(Word, p.lay.rsize[RG_REC] - p.lay.jm_off)
-            for (int w = 0; w < W32; ++w) nact -= __popc(FG_AT(R.allm, w, FG_N(uint32_t, p.lay.rsize[RG_ALL])));
+            for (int w = 0; cs1 > cs0 && w < W32; ++w) nact -= __popc(FG_AT(R.allm, w, FG_N(uint32_t, p.lay.rsize[RG_ALL])));
             for (int j = ltid; j <= n2; j += LT) {
                 int pos = j;
                 bool fr = true;
