@@ -789,8 +789,10 @@ static int tune_class(fastged_handle *h, ClassPlan &cp, int B, int forced_block,
     const bool tuned = forced_block == 0 &&
                        tune_lookup(class_key(cp, B, npairs, h->sm_count), &tc);
     if (tuned) forced_block = tc.block;
+    bool by_rule = false;
     if (cluster_eligible(cp, npairs, h->sm_count)) {
         const char *env = getenv("FASTGED_CLUSTER");
+        by_rule = !env && !forced_cluster && !tuned;
         int cl = env ? atoi(env)
                      : forced_cluster ? forced_cluster
                                       : (tuned ? tc.cluster : cluster_rule(cp, npairs, h->sm_count));
@@ -798,15 +800,20 @@ static int tune_class(fastged_handle *h, ClassPlan &cp, int B, int forced_block,
             cp.cluster = cl;
         }
     }
-    if (cp.cluster > 1) {
+    // a size of the built-in rule that the GPU cannot hold (16 CTAs need that many free SMs in
+    // one GPC) is halved until one fits; a size asked for is reported instead
+    for (; cp.cluster > 1; cp.cluster >>= 1) {
         plan_layout(cp, B, forced_block ? forced_block : 512, max_dyn);
         const int block = cp.block = forced_block ? forced_block : 512;
         int nclu = 0;
         cudaError_t e = kbest_cluster_occupancy(cp.W, cp.wide, label_instance(B), block,
                                                 (size_t)cp.lay.smem_bytes, cp.cluster, &nclu);
+        if (by_rule && (e != cudaSuccess || nclu < 1)) {
+            cudaGetLastError();
+            continue;
+        }
         if (e != cudaSuccess) return cuda_fail(e, "cluster occupancy query");
         if (nclu < 1) return set_error(FASTGED_ERR_CUDA, "a cluster team does not fit the GPU");
-        cp.block = block;
         cp.smem = (size_t)cp.lay.smem_bytes;
         cp.all_smem = false;
         cp.grid = std::min(nclu, npairs) * cp.cluster;

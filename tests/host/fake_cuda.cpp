@@ -268,10 +268,14 @@ cudaError_t kbest_occupancy(int, bool, bool, bool, int, int, size_t, int *out)
     *out = 2;
     return cudaSuccess;
 }
+// clusters of more than g_max_cluster CTAs do not fit (or, with g_cluster_error, the query fails)
+static std::atomic<int> g_max_cluster{16};
+static std::atomic<bool> g_cluster_error{false};
 cudaError_t kbest_cluster_occupancy(int, bool, int, int, size_t, int cluster, int *out)
 {
-    *out = 152 / cluster;
-    return cudaSuccess;
+    const bool fits = cluster <= g_max_cluster.load();
+    *out = fits ? 152 / cluster : 0;
+    return fits || !g_cluster_error.load() ? cudaSuccess : cudaErrorInvalidValue;
 }
 // one-warp launches report their vertex-map placement as cluster 100 + gmap
 cudaError_t launch_kbest_warp(bool, int, const KParams &p, int, int block, size_t, cudaStream_t)
@@ -303,3 +307,10 @@ extern "C" int fake_max_pack_graphs(int reset)
 
 // the next n packing launches fail (a batch's launch error)
 extern "C" void fake_fail_launches(int n) { fastged::g_fail_launches.store(n); }
+
+// clusters of more than n CTAs do not fit the GPU; with error, the query reports one for them
+extern "C" void fake_set_max_cluster(int n, int error)
+{
+    fastged::g_max_cluster.store(n);
+    fastged::g_cluster_error.store(error != 0);
+}
