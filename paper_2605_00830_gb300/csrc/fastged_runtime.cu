@@ -713,11 +713,13 @@ static bool team_beats_warps(const ClassPlan &cp, int n_pairs, int sm_count)
 // levels are too small (K = 32: 18.7 and 17.9 ms). Otherwise about 20,000 successors per CTA,
 // between 2 and 8 CTAs, halved while the class's teams would take more than two waves of the
 // GPU (smaller teams spend fewer cluster barriers per successor; 16 pairs at K = 100,000: 12.3
-// ms on 8 CTAs, 16.0 ms on 16).
-static int cluster_rule(const ClassPlan &cp, int npairs, int sm_count)
+// ms on 8 CTAs, 16.0 ms on 16). Under a cap of max_sms SMs the 16 have to fit those: a cap of 8
+// must not give one pair 16.
+static int cluster_rule(const ClassPlan &cp, int npairs, int sm_count, int max_sms)
 {
     const int64_t succ = (int64_t)cp.kmax * (cp.n2max + 1);
-    if ((int64_t)npairs * 16 <= sm_count && succ >= (cp.W >= 8 ? 400000 : 16384)) return 16;
+    const int sms = max_sms > 0 ? std::min(max_sms, sm_count) : sm_count;
+    if ((int64_t)npairs * 16 <= sms && succ >= (cp.W >= 8 ? 400000 : 16384)) return 16;
     int cl = succ <= 40000 ? 2 : succ <= 160000 ? 4 : 8;
     while (cl > 2 && (int64_t)npairs * cl > 2 * (int64_t)sm_count) cl >>= 1;
     return cl;
@@ -793,9 +795,10 @@ static int tune_class(fastged_handle *h, ClassPlan &cp, int B, int forced_block,
     if (cluster_eligible(cp, npairs, h->sm_count)) {
         const char *env = getenv("FASTGED_CLUSTER");
         by_rule = !env && !forced_cluster && !tuned;
-        int cl = env ? atoi(env)
-                     : forced_cluster ? forced_cluster
-                                      : (tuned ? tc.cluster : cluster_rule(cp, npairs, h->sm_count));
+        int cl = env              ? atoi(env)
+                 : forced_cluster ? forced_cluster
+                 : tuned          ? tc.cluster
+                                  : cluster_rule(cp, npairs, h->sm_count, max_sms);
         if (cl == 1 || cl == 2 || cl == 4 || cl == 8 || cl == 16) {
             cp.cluster = cl;
         }

@@ -41,3 +41,12 @@ def test_a_cluster_asked_for_is_refused_when_it_does_not_fit(lib):
     mm = F.Marshalled(w.graphs, w.pairs)
     o = F.make_options(team=F.FASTGED_TEAM_CTA, cluster=16)
     assert lib.probe_flatten(ctypes.addressof(mm.pl), 5000, ctypes.addressof(o), c) == F.FASTGED_ERR_CUDA
+
+
+@pytest.mark.parametrize("max_sms,cluster,grid", [(0, 16, 48), (152, 16, 48), (48, 16, 48),
+                                                  (47, 8, 24), (16, 8, 16), (8, 8, 8), (4, 8, 8)])
+def test_sixteen_ctas_per_pair_stay_within_the_cap(lib, max_sms, cluster, grid):
+    """Three pairs of one class; the sizes of eight CTAs and less are the rule's for any cap."""
+    w = W.config4(3, n_range=(600, 700))
+    (c,) = _probe_classes(lib, w, 1024, full=True, max_sms=max_sms)
+    assert (c["cluster"], c["grid"]) == (cluster, grid)
