@@ -689,20 +689,36 @@ static bool cluster_eligible(const ClassPlan &cp, int npairs, int sm_count)
     return cp.W >= 4 || (int64_t)cp.kmax * (cp.n2max + 1) >= 16384;
 }
 
+// What one pair of a one-warp class would gain from a CTA: the successors its warp scores in the
+// rounds of 32 nodes after the first, over all levels. None for beams below 64 nodes and for
+// short sources, where a CTA's barriers per level cost more.
+static int64_t team_gain(int n1, int n2, int K)
+{
+    return K >= 64 && n1 >= 16 ? (int64_t)(K - 32) * n1 * (n2 + 1) : 0;
+}
+
 // A batch of few pairs leaves most warps of the GPU without one, and takes as long as one warp
-// needs for its largest pair: a CTA per pair is then faster. Measured at K = 100 on pairs of
-// 10-40 vertices, whole calls, one-warp and 256-thread teams: 1 pair 201 and 138 us, 100 pairs
-// 571 and 320, 500 pairs 626 and 412, 1,001 pairs 688 and 597, 2,000 pairs 878 and 952; up to
-// 14 vertices 500 pairs 177 and 202. At K = 16 one warp is the faster one for any number (100
-// pairs: 204 and 263). A class whose one-warp shapes are being timed stays with them (its
-// sample is smaller than the batch it stands for).
-static bool team_beats_warps(const ClassPlan &cp, int n_pairs, int sm_count)
+// needs for its heaviest pair: a CTA per pair is then faster. The CTAs' own cost is a share of
+// an SM per level, so the largest gain of a pair is compared with a fixed cost and the levels
+// per SM. Fitted to 471 measured batches (whole calls, K 16-128 and mixed, pairs of 5-60
+// vertices, 1-1,600 of them, 8-152 SMs); one-warp and CTA teams in us, 10-40 vertices: K = 100,
+// 152 pairs 588 and 327, 800 pairs 680 and 494, 1,216 pairs 730 and 669, 1,600 pairs 774 and
+// 804; K = 64, 400 pairs 428 and 352, 800 pairs 485 and 533; K = 100, 1,000 pairs of 14-20
+// vertices 326 and 402; K = 32 with one pair of 64, 500 pairs 321 and 389. A cap on the SMs
+// counts for two and a half times its SMs (the CTAs of such batches do not fill theirs): K =
+// 100, 16 SMs, 200 pairs 576 and 397, 600 pairs 648 and 981; 50 SMs, 600 pairs 654 and 507. A
+// class whose one-warp shapes are being timed stays with them (its sample is smaller than the
+// batch it stands for).
+static bool team_beats_warps(const ClassPlan &cp, int n_pairs, int sm_count, int max_sms)
 {
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
         if (g_tune_forcing && g_tune_force.gmap >= 0) return false;
     }
-    return cp.kmax >= 64 && cp.n1max >= 16 && n_pairs <= 8 * sm_count;
+    // SMs in halves
+    const int64_t s2 = max_sms > 0 ? std::min<int64_t>(5 * (int64_t)max_sms, 2 * (int64_t)sm_count)
+                                   : 2 * (int64_t)sm_count;
+    return n_pairs <= 8 * sm_count && cp.gain * s2 >= 12000 * s2 + 760 * cp.levels;
 }
 
 // CTAs per cluster without a tuning entry. A handful of pairs (16 CTAs each still fit the GPU
@@ -1077,6 +1093,7 @@ int fastged::flatten(fastged_handle *h, const fastged_pair_list *pl, int32_t K,
         int8_t W = 1, wide = 0, w32 = 0, pk = 0, warp = 0;
         int n1max = 0, n2max = 0, m1max = 0, kmax = 1;
         int bmin = kBuckets, bmax = -1;
+        int64_t levels = 0, gain = 0;   // one-warp classes: see ClassPlan
     };
     struct PairChunk {
         int64_t maps = 0;                // map entries of the chunk, then its base offset
@@ -1142,6 +1159,10 @@ int fastged::flatten(fastged_handle *h, const fastged_pair_list *pl, int32_t K,
             kc.kmax = std::max(kc.kmax, kp);
             kc.bmin = std::min(kc.bmin, bk);
             kc.bmax = std::max(kc.bmax, bk);
+            if (warp) {
+                kc.levels += g1.n;
+                kc.gain = std::max(kc.gain, team_gain(g1.n, g2.n, kp));
+            }
             C.maps += g1.n;
         }
     });
@@ -1170,6 +1191,8 @@ int fastged::flatten(fastged_handle *h, const fastged_pair_list *pl, int32_t K,
                 y.kmax = std::max(y.kmax, x.kmax);
                 y.bmin = std::min(y.bmin, x.bmin);
                 y.bmax = std::max(y.bmax, x.bmax);
+                y.levels += x.levels;
+                y.gain = std::max(y.gain, x.gain);
             }
         int keys[kKeys], nk = 0;
         for (int k = 0; k < kKeys; ++k) {
@@ -1191,6 +1214,8 @@ int fastged::flatten(fastged_handle *h, const fastged_pair_list *pl, int32_t K,
             cp.m1max = y.m1max;
             cp.n2max = y.n2max;
             cp.kmax = y.kmax;
+            cp.levels = y.levels;
+            cp.gain = y.gain;
             int32_t run = 0;
             for (int bk = y.bmin; bk <= y.bmax; ++bk)
                 for (PairChunk &C : pcs) {
@@ -1211,7 +1236,7 @@ int fastged::flatten(fastged_handle *h, const fastged_pair_list *pl, int32_t K,
     }
     b.map_total = mtot;
     for (auto &cp : b.classes) {
-        if (cp.warp && team_beats_warps(cp, np, h->sm_count)) cp.warp = false;
+        if (cp.warp && team_beats_warps(cp, np, h->sm_count, opt.max_sms)) cp.warp = false;
         int rc = tune_class(h, cp, B, opt.block_threads, opt.max_sms, opt.cluster);
         if (rc) return rc;
     }

@@ -46,6 +46,7 @@ struct ClassPlan {
     bool warp = false;            // one warp per pair (kbest_warp_kernel; W == 1, small K)
     WarpLayout wl{};              // layout of one warp's working set (warp classes)
     int n1max = 0, n2max = 0, m1max = 0, kmax = 1;
+    int64_t levels = 0, gain = 0; // one-warp classes: sum of n1, largest team_gain of a pair
     std::vector<int32_t> order;   // pair indices, heaviest first
     int64_t order_off = 0;        // offset of this class's order in the device order array
     Layout lay{};

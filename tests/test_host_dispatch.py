@@ -5,6 +5,7 @@ caller asks for are reported when they cannot.
 """
 import ctypes
 
+import numpy as np
 import pytest
 
 from host_probe import load
@@ -50,3 +51,47 @@ def test_sixteen_ctas_per_pair_stay_within_the_cap(lib, max_sms, cluster, grid):
     w = W.config4(3, n_range=(600, 700))
     (c,) = _probe_classes(lib, w, 1024, full=True, max_sms=max_sms)
     assert (c["cluster"], c["grid"]) == (cluster, grid)
+
+
+def _paths(sizes, n_pad=0):
+    """Pairs of equal path graphs of the given sizes, and n_pad pairs of 70-vertex ones."""
+    g = [W.Graph(n, np.zeros(n, np.int32), np.stack([np.arange(n - 1), np.arange(1, n)], 1).astype(np.int32))
+         for n in list(sizes) + [70] * n_pad]
+    return W.Workload("paths", g, np.repeat(np.arange(len(g), dtype=np.int32), 2).reshape(-1, 2),
+                      W.UNIT_COSTS, 128)
+
+
+def _warps(lib, w, K, **opts):
+    """Whether the batch's single-word class of at most 31 target vertices takes one-warp teams."""
+    cls = _probe_classes(lib, w, K, team=F.FASTGED_TEAM_AUTO, full=True, **opts)
+    (c,) = [c for c in cls if c["n2max"] <= 31]
+    return bool(c["warp"])
+
+
+# one CTA per pair while the largest gain of a pair, (K - 32) n1 (n2 + 1), is at least
+# 12,000 + 380 levels per SM; by hand for the 152 SMs of the fakes
+@pytest.mark.parametrize("n,K,opts,most", [
+    (20, 100, {}, 331),                  # 68 * 420 = 28,560: 16,560 * 152 / (380 * 20) = 331.2
+    (20, 64, {}, 28),                    # 32 * 420 = 13,440:  1,440 * 152 / 7,600 = 28.8
+    (20, 63, {}, 0), (15, 128, {}, 0),   # below 64 nodes or 16 source vertices: never
+    (31, 128, {}, 1073),                 # 96 * 992 = 95,232: 83,232 * 152 / 11,780 = 1,073.9
+    (20, 100, {"max_sms": 10}, 54),      # 25 SMs: 16,560 * 25 / 7,600 = 54.5
+    (20, 100, {"max_sms": 1}, 5),        # 2.5 SMs: 5.4
+    (20, 100, {"max_sms": 100}, 331)])   # 250 SMs: no more than there are
+def test_few_pairs_take_a_cta_each(lib, n, K, opts, most):
+    if most:
+        assert not _warps(lib, _paths([n] * most), K, **opts)
+    assert _warps(lib, _paths([n] * (most + 1)), K, **opts)
+
+
+def test_the_largest_gain_decides_and_the_batch_bounds_it(lib):
+    # 100 pairs, 2,000 levels: 12,000 + 5,000. One K = 64 among K = 32 gains 13,440, one K = 100
+    # 28,560
+    w = _paths([20] * 100)
+    for top, warps in ((32, True), (64, True), (100, False)):
+        kpp = np.full(100, 32, np.int32)
+        kpp[57] = top
+        assert _warps(lib, w, 128, k_per_pair=kpp) == warps
+    # batches of more than 8 * 152 pairs keep their one-warp classes
+    for pad, warps in ((1116, False), (1117, True)):
+        assert _warps(lib, _paths([20] * 100, pad), 100) == warps
