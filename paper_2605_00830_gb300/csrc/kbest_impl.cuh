@@ -496,7 +496,11 @@ __device__ __forceinline__ void score_table(const KParams &p, const Regions<Word
     }
 }
 
-// Scores this warp's nodes again for the exact selection (the node vectors are in place).
+// Scores this warp's nodes again for the exact selection (the node vectors are in place). A warp
+// without nodes must not enter the scoring, which reads a column's tables before its first node:
+// the CTA may have none at all, and then no list of columns. (The test stands here and not in
+// solve_pair's column count, where two more conditions cost two-word clusters 15 %: 16 wide
+// beams 13.1 -> 15.0 ms.)
 template <int W, typename Word, int BK>
 __device__ __noinline__ void score_exact(const KParams &p, const Regions<Word> &R,
                                          const LevelView<Word> &V, int B, int n2, int nw,
@@ -505,6 +509,7 @@ __device__ __noinline__ void score_exact(const KParams &p, const Regions<Word> &
     const int lane = threadIdx.x & 31;
     for (int b = lane; b < kBuckets; b += 32) FG_AT(hrow, b, kBuckets) = 0;
     __syncwarp();
+    if (V.s_lo >= V.s_hi) return;
     if (p.cost.eins == p.cost.edel)
         score_nodes<W, Word, BK, true, true>(p, R, V, B, n2, nw, V.s_lo, V.s_hi - V.s_lo, anchor, sh, hrow);
     else
@@ -1033,16 +1038,16 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
             if (lane < W32) atomicAnd(&FG_AT(R.allm, lane, FG_N(uint32_t, p.lay.rsize[RG_ALL])), am);
         }
         __syncthreads();
-        // active columns, increasing: the vertices not used by all, and the deletion n2. None
-        // for a cluster CTA without nodes (levels of fewer nodes than CTAs): its used-by-all mask
-        // is still all ones and its column list is not written, so no pass may read it
-        int nact = cs1 > cs0 ? n2 + 1 : 0, stride;
+        // active columns, increasing: the vertices not used by all, and the deletion n2. A
+        // cluster CTA without nodes (levels of fewer nodes than CTAs) has no such list: its
+        // mask is still all ones, its count means nothing, and score_exact does not read them
+        int nact = n2 + 1, stride;
         {
             using Rec = ColRec<Word, (BK == 8 ? kMaxB : BK)>;
             constexpr int NPL = BK == 8 ? kMaxB : BK;
             Word *jm = (Word *)((uint8_t *)R.rec + p.lay.jm_off);   // one-hot vertex bits
 #define NJM FG_N(Word, p.lay.rsize[RG_REC] - p.lay.jm_off)
-            for (int w = 0; cs1 > cs0 && w < W32; ++w) nact -= __popc(FG_AT(R.allm, w, FG_N(uint32_t, p.lay.rsize[RG_ALL])));
+            for (int w = 0; w < W32; ++w) nact -= __popc(FG_AT(R.allm, w, FG_N(uint32_t, p.lay.rsize[RG_ALL])));
             for (int j = ltid; j <= n2; j += LT) {
                 int pos = j;
                 bool fr = true;
