@@ -92,7 +92,7 @@ enum WarpRegion : int {
 // label planes and the 32-bit cost-row entry, padded to 16 bytes (vector loads)
 constexpr int warp_rec_bytes(bool w32, int npl)
 {
-    return ((w32 ? 4 : 8) * (1 + npl) + 4 + 15) / 16 * 16;
+    return ((w32 ? 4 : 8) * (1 + npl) + 15) / 16 * 16;
 }
 
 // bytes of one column record of the single-word teams (ColRec): adjacency word, label planes

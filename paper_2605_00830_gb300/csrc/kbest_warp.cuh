@@ -47,18 +47,16 @@ constexpr int kWarpChunks = 4;
 constexpr int kWarpPadCost = 1 << 24;
 
 // Target record of g2 vertex u at index u, or of the deletion column at index n2 (no
-// neighbours, no labels): adjacency word and NPL edge-label planes. (ColRec, one per active
+// neighbours, no labels): adjacency word and NPL edge-label planes. (WarpRec, one per active
 // column of a level, also holds the cost entry.)
 template <typename Word, int NPL>
 struct __align__(16) TgtRec {
     Word a2;
     Word l[NPL];
-    int32_t crow;
 };
 template <typename Word>
 struct __align__(16) TgtRec<Word, 0> {
     Word a2;
-    int32_t crow;
 };
 
 static_assert(sizeof(TgtRec<uint32_t, 0>) == warp_rec_bytes(true, 0), "record size");
@@ -476,7 +474,6 @@ __device__ __forceinline__ void solve_pair_warp(const KParams &p, uint32_t wb, u
                                         ? (Word)FG_AT(pl2, ((int64_t)b * n2 + u) * W2,
                                                       p.plane_words - m2.plane_off)
                                         : (Word)0);
-            r.crow = 0;
             FG_AT(R.tgt(wl), u, WN(Rec, WR_TGT)) = r;
             if (vtx)
                 FG_AT(R.lab2(wl), u, WN(int32_t, WR_LAB2)) =
