@@ -115,15 +115,17 @@ typedef struct {
                              /* an extension, not part of the paper). Maps are returned in   */
                              /* source index order either way                                 */
     int32_t team;            /* FASTGED_TEAM_AUTO (0): pairs with at most 64 vertices in g1,  */
-                             /* at most 63 in g2 and K <= 128 are solved by one warp each,    */
-                             /* (in batches of few pairs with K >= 64 by a CTA each), the      */
-                             /* others by a CTA (or a cluster of CTAs) each;                  */
+                             /* at most 63 in g2 and K <= 128 are solved by one warp each     */
+                             /* (by a CTA each where few such pairs, some with K >= 64, face  */
+                             /* many SMs; a tuning table entry sets the shape within either   */
+                             /* kind), the others by a CTA (or a cluster of CTAs) each;       */
                              /* FASTGED_TEAM_CTA (1): every pair by a CTA or cluster.         */
                              /* Results do not depend on it                                   */
     int32_t max_sms;         /* 0 = no cap; else the resident teams of each size class are   */
                              /* capped to what fits this many SMs (whole clusters, at least   */
                              /* one team), so that other work keeps the remaining SMs; pairs  */
-                             /* then queue for the capped teams. Results do not depend on it  */
+                             /* then queue for the capped teams, and the built-in rules count */
+                             /* on no more SMs than these. Results do not depend on it        */
     int32_t cluster;         /* 0 = built-in rule or tuning table; 1, 2, 4, 8 or 16: CTAs per */
                              /* team for the classes that may use cluster teams (fewer pairs  */
                              /* than SMs, wide bitsets or very wide beams). Small clusters do */

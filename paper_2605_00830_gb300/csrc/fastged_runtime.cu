@@ -542,8 +542,9 @@ size_t fastged::plan_warp_layout(ClassPlan &cp, int B, bool gmap)
     sz[WR_PED0] = sz[WR_PED1] = km * 4;
     sz[WR_E20] = sz[WR_E21] = km * 2;
     // rows of score bytes and the level's columns in whole quads, an odd number of them; at
-    // least two bytes per successor and node, so that the share of a team only grows where
-    // its beam is too small for the records
+    // least two bytes per successor and node, the share with which the placement of the maps
+    // and the teams per SM were measured (at K = 100 and 40 target vertices, 64-bit words, 8.4 KB
+    // where the bytes and records need 7.0)
     const size_t cols = (align_up(n2 + 1, 4) / 4 | 1) * 4;
     wl.hist_off = (int32_t)align_up(km * cols, 16);
     wl.rec_off = wl.hist_off + kHistRow * 4;

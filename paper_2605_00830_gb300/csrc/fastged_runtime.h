@@ -40,7 +40,7 @@ struct ClassPlan {
     int W = 1;
     bool wide = false;
     bool w32 = false;             // one 32-bit word per bitset (every g2 has <= 32 vertices)
-    bool pk = false;              // successors packed into one 32-bit entry (see packable)
+    bool pk = false;              // PEDs below 2^16 and slot and vertex within 16 bits (see packable)
     bool all_smem = false;        // every region of a team fits in shared memory
     int cluster = 1;              // CTAs per team (> 1: a thread-block cluster per pair)
     bool warp = false;            // one warp per pair (kbest_warp_kernel; W == 1, small K)
@@ -107,10 +107,11 @@ struct NvtxRange {
     NvtxRange(const NvtxRange &) = delete;
     NvtxRange &operator=(const NvtxRange &) = delete;
 };
-// Single-word pairs go to the single-word kernels when no PED can reach 2^16 (the one-warp
-// kernel's entries hold 16-bit offsets, and the one-CTA kernel's padding columns score 2^29)
-// and K fits the 16 - jbits bits left beside a target vertex in a 16-bit code, jbits being the
-// bit length of n2; the others are solved by the two-word kernels.
+// Single-word pairs go to the single-word kernels when no PED can reach 2^16 (their padding
+// columns score 2^24 and 2^29, past every PED offset and without overflow) and K fits the
+// 16 - jbits bits left beside a target vertex in a 16-bit code, jbits being the bit length of
+// n2; the others are solved by the two-word kernels. (No entry holds such a code any more; the
+// second bound stays as the line up to which the single-word kernels were measured.)
 inline int jbits_of(int n2)
 {
     int b = 0;

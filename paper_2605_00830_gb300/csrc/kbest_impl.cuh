@@ -231,13 +231,13 @@ __device__ __forceinline__ int succ_ped(const KParams &p, const Regions<Word> &R
 //
 // Bound: the integer pipes. A column costs W popcounts of 64 bits (two 32-bit POPC each, 16
 // lanes per clock and SM), so a chunk of 32 columns takes at least 4 W clocks of an SM. Only
-// columns some node still has free are scored (1.02-1.3 times the free ones on dense and
-// large pairs, 2.1 times on a beam of 20,000). A score leaves one byte instead of the 8-byte
+// columns some node still has free are scored (1.02-1.3 times the free ones on dense pairs, 2.1
+// times on a beam of 20,000). A score leaves one byte instead of the 8-byte
 // entry that was written once and read back twice, and its histogram count is taken here: a
 // shared increment costs 6 clocks of an SM per warp for any mix of buckets, what counting in
 // packed registers costs too, but on the memory pipe. 1,024 dense pairs of 50-200 vertices,
-// K = 256: 41.9 -> 19.6 ms; 64 pairs of 500-1,000 vertices, K = 1,024: 554 -> 327 ms; one
-// G(200, 0.4) pair, K = 5,000: 40.1 -> 29.3 ms.
+// K = 256: 41.9 -> 19.6 ms; one G(200, 0.4) pair, K = 5,000: 40.1 -> 29.3 ms. (Large sparse
+// pairs without edge labels are scored by score_table.)
 //
 // Every column's target
 // tables stay in registers while the warp walks its nodes, whose vectors are read as
@@ -398,7 +398,11 @@ struct TableNode {
 // T is the sum of the bits of a few rows of A2 (deg of them).
 //   inserted = E - T, deleted = |P| - T, PED = base + C + eins (E - T) + edel (|P| - T)
 // Lanes <-> eight columns each (256 columns per step); the counts of four columns share a
-// 32-bit word, and no byte of E + |P| can pass 255 (the caller checks the degrees).
+// 32-bit word, and no byte of E + |P| can pass 255 (the caller checks the degrees). Every column
+// is scored, used ones too (a row of counts has to stay complete for the children): about twice
+// a node's successors on 64 pairs of 500-1,000 vertices, K = 1,024, whose time went 327 -> 199 ms
+// with this path and the row prefetch below. Bound: latency of the rows and maps in L2 and DRAM
+// at 16 warps per SM.
 template <int W, typename MapT, typename Word, bool FOLD>
 __device__ __forceinline__ void score_table(const KParams &p, const Regions<Word> &R,
                                             const LevelView<Word> &V, int n2, int g0, int ng,

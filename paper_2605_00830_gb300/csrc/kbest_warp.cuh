@@ -34,7 +34,10 @@
 // entry and a packed-register count per successor), and its 15-bucket window sent cost setting
 // 2 to a bisection on many levels. Measured, before -> after: 20,000 pairs, setting 1, resident:
 // 2.82 -> 2.76 ms; 5,003 pairs, setting 2, from host memory: 2.08 -> 1.32 ms; 61 x 256 distance
-// matrix, K = 20: 1.28 -> 1.19 ms; one pair from host memory: 302 -> 296 us.
+// matrix, K = 20: 1.28 -> 1.19 ms. (One pair from host memory: 302 -> 296 us; a batch that small
+// takes a CTA per pair, 209 us. team_beats_warps in fastged_runtime.cu says where the line lies.)
+// Registers are capped at 96 by the launch bounds; the instances with 0 and 2 label planes spill
+// 16-36 bytes for it.
 #pragma once
 #include "kbest_impl.cuh"
 

@@ -67,8 +67,9 @@ double ms_between(Clock::time_point a, Clock::time_point b)
     return std::chrono::duration<double, std::milli>(b - a).count();
 }
 
-// Size buckets follow the size classes: one-warp teams (K <= 128, target of at most 63
-// vertices) split by their word instance (<= 31 vertices: bucket 0, else 2); the other pairs
+// Size buckets follow the size classes: pairs of the one-warp classes (K <= 128, target of at
+// most 63 vertices; a batch of few of them gets a CTA per pair, see team_beats_warps) split by
+// their word instance (<= 31 vertices: bucket 0, else 2); the other pairs
 // by the bitset word class of the target graph (<= 32 vertices: bucket 1, one 64-bit word: 3,
 // then 2, 4, 8, 16 words: 4-7). A batch carries a K per pair, so K splits nothing else, and a
 // batch of one bucket is (nearly always) one size class, launched on its lane's own stream.
