@@ -45,9 +45,9 @@ os.environ.setdefault("CUDA_DEVICE_MAX_CONNECTIONS", "32")
 KERNEL_SOURCES = ["kbest_impl.cuh", "kbest_warp.cuh", "kbest_kernels.cu", "kbest_b0.cu",
                   "kbest_b2.cu", "kbest_b8.cu", "fastged_internal.h"]
 CAPTURED_TRAFFIC = {
-    # both one-warp launches of the 20,000-pair step (4-warp CTAs): 38.9 + 54.7 MB, cold cache
-    "molecule": {"bytes_per_step": 93652736,
-                 "sources_sha256": "348c17fdbef3c72a0e8d7dffd0eeebdb9a149a1d142427fd523f2855ffe81b04"},
+    # both one-warp launches of the 20,000-pair step (4-warp CTAs): 39.1 + 54.9 MB, cold cache
+    "molecule": {"bytes_per_step": 93988864,
+                 "sources_sha256": "046ab2228b2b232c650caf9c4997d262dc27b1dd731277308a9292d469f6e1b4"},
 }
 
 
@@ -241,15 +241,41 @@ def int_ops_per_eval(W: int, B: int, fold: bool) -> int:
     return (word + lab) * W + 6
 
 
+def int_ops_per_counted(mean_deg: float, fold: bool) -> float:
+    """The same for a successor scored from rows of neighbour counts. Per 32-bit word of four
+    columns: the parent's count plus a row of bits (2 ops), such a row for each prior neighbour
+    of v_i (2 ops each, mean_deg on average) and their combination (3 ops, or 1 with two-term
+    costs); per column the extraction of one byte (2 ops) or two (4), the used-bit test and the
+    cost sum (6)."""
+    return (2 + 2 * mean_deg + (3 if fold else 1)) / 4 + (2 if fold else 4) + 6
+
+
+def counted_pairs(w, mm):
+    """Pairs scored from rows of neighbour counts: targets of more than 256 vertices, no edge
+    labels, at most eight prior neighbours per source vertex on average, no degree above 127."""
+    lab = np.array([g.elabel is not None and g.m > 0 and int(np.max(g.elabel)) > 0 for g in w.graphs])
+    m = np.array([g.m for g in w.graphs], np.int64)
+    deg = np.array([int(np.bincount(np.asarray(g.edges).ravel()).max()) if g.m > 0 else 0
+                    for g in w.graphs])
+    prior = np.array([int(np.bincount(np.asarray(g.edges).max(axis=1)).max()) if g.m > 0 else 0
+                      for g in w.graphs])
+    a, d = np.asarray(mm.pairs)[:, 0], np.asarray(mm.pairs)[:, 1]
+    return ((mm.n[d] > 256) & ~lab[a] & ~lab[d] & (m[a] <= 8 * mm.n[a]) & (deg[d] <= 127) &
+            (prior[a] <= 127)), m[a]
+
+
 def algorithmic_work(w, mm, n_out):
     """(integer ops, substitution successors, algorithmic HBM bytes) of one pass over w.
 
     Integer ops: each pair's substitution successors (deletions and completions do no bitset
     work; every level expands at most K nodes with one deletion child each, so this count is
-    a lower bound) times the 32-bit operations of one evaluation for that pair's bitset words.
+    a lower bound) times the 32-bit operations of one evaluation for that pair's bitset words,
+    or of one from its rows of counts.
     HBM bytes, per pair: both graphs' bitsets (W words per row, 1 + b planes) and labels, the
     cost and map written back, and for classes whose beam lives in global memory the beam
-    state of every level (2 K (2 n1 + 8 W + 16) bytes) plus 8 bytes per scored successor."""
+    state of every level (2 K (2 n1 + 8 W + 16) bytes) plus a score byte per successor, written
+    and read, and for pairs with rows of counts a row of n2 + 1 bytes per kept node and level,
+    written and read."""
     fold = w.cost[4] == w.cost[5]
     B = 0
     labs = [int(gr.elabel.max()) for gr in w.graphs if gr.elabel is not None and gr.m > 0]
@@ -260,19 +286,22 @@ def algorithmic_work(w, mm, n_out):
     K = (np.asarray(w.k_per_pair, np.int64) if w.k_per_pair is not None
          else np.full(mm.n_pairs, w.K, np.int64))
     subs = np.maximum(n_out - (n1s + 1) * K, 0)
+    counted, m1s = counted_pairs(w, mm)
     ops = 0
     for p_w, sel in ((0, n2s <= 32), (1, (n2s > 32) & (n2s <= 64)), (2, (n2s > 64) & (n2s <= 128)),
                      (4, (n2s > 128) & (n2s <= 256)), (8, (n2s > 256) & (n2s <= 512)),
                      (16, n2s > 512)):
-        ops += int_ops_per_eval(p_w, B, fold) * int(subs[sel].sum())
+        ops += int_ops_per_eval(p_w, B, fold) * int(subs[sel & ~counted].sum())
+    ops += int(sum(int_ops_per_counted(m / max(n, 1), fold) * s
+                   for m, n, s in zip(m1s[counted], n1s[counted], subs[counted])))
     W1 = (n1s + 63) // 64
     W2 = (n2s + 63) // 64
     io = (n1s * (8 * W1 * (1 + B) + 1) + n2s * (8 * W2 * (1 + B) + 1) + 4 * (1 + n1s)).sum()
     # beams in global memory: pairs of more than 128 target vertices, or beams of more than
-    # 2^16 successors per level (the cluster teams' regime)
+    # 2^16 successors per level
     spill = (n2s > 128) | (K * (n2s + 1) >= 65536)
     beam = (n1s * 2 * np.minimum(K, 1 + n1s * n2s) * (2 * n1s + 8 * W2 + 16))[spill].sum()
-    cand = 8 * n_out[spill].sum()
+    cand = 2 * n_out[spill].sum() + (n1s * 2 * K * (n2s + 1))[counted].sum()
     return ops, int(subs.sum()), int(io + beam + cand), bool(spill.any())
 
 
