@@ -193,6 +193,12 @@ struct LevelView {
     int nact;               // active columns of the level
     int stride;             // bytes per row of score bytes (>= nact)
     int64_t nimg;           // elements behind imgw
+    // eight and more words: the level's rows of neighbour counts (null: none are kept), the
+    // beam's maps and their stride, v_i's prior neighbours in the list
+    const uint8_t *et;
+    const uint16_t *map;
+    int64_t mt;
+    int n0, deg;
 };
 
 // PED of successor (node s, column j). Column j == n2 is the deletion v_i -> eps: its A2
@@ -227,6 +233,14 @@ __device__ __forceinline__ int succ_ped(const KParams &p, const Regions<Word> &R
            FG_AT(V.crow, j, N2S) + p.cost.eins * x + p.cost.edel * y + p.cost.esub * z;
 }
 
+// Score byte of PED offset d in a pass of the exact selection: with sh > 0 in units of 2^sh,
+// offsets below 0 left out; sh == 0 gives 0 below 0 and 1 + d from there on.
+__device__ __forceinline__ int exact_byte(int d, int sh)
+{
+    if (sh > 0) return d < 0 ? kScoreMax : min(d >> sh, kScoreMax);
+    return d < 0 ? 0 : min(d, kScoreMax - 1) + 1;
+}
+
 // S3 over nodes [g0, g0 + ng) of this warp, lanes <-> active columns.
 //
 // Bound: the integer pipes. A column costs W popcounts of 64 bits (two 32-bit POPC each, 16
@@ -245,8 +259,7 @@ __device__ __forceinline__ int succ_ped(const KParams &p, const Regions<Word> &R
 // one byte and one count in the warp's histogram row (a shared-memory increment, which the
 // hardware aggregates over lanes with the same bucket).
 // EXACT = 0: offset from `anchor`, offsets below it counting as 0. EXACT = 1 (selection
-// past the histogram window): sh >= 0 gives (PED - anchor) >> sh with PEDs below the anchor
-// left out; sh < 0 marks 0 = below the anchor, 1 = at the anchor, 127 = above.
+// past the histogram window): see exact_byte.
 template <int W, typename Word, int BK, bool FOLD, bool EXACT>
 __device__ __forceinline__ void score_nodes(const KParams &p, const Regions<Word> &R,
                                             const LevelView<Word> &V, int B, int n2, int nw,
@@ -311,12 +324,8 @@ __device__ __forceinline__ void score_nodes(const KParams &p, const Regions<Word
             const uint32_t uw = FG_AT((const uint32_t *)V.imgw, im * (int)(sizeof(Word) / 4) + jw,
                                       V.nimg * (int)(sizeof(Word) / 4));
             int v;
-            if (EXACT) {
-                if (sh >= 0) v = d < 0 ? kScoreMax : min(d >> sh, kScoreMax);
-                else v = d < 0 ? 0 : d == 0 ? 1 : kScoreMax;
-            } else {
-                v = max(0, min(d, kScoreMax));
-            }
+            if (EXACT) v = exact_byte(d, sh);
+            else v = max(0, min(d, kScoreMax));
             if (uw & jm) v = kScoreMax;
             if (ok) {
                 FG_AT(R.score, (int64_t)(s - V.cs0) * V.stride + a, FG_N(uint8_t, p.lay.rsize[RG_SCORE])) = (uint8_t)v;
@@ -500,6 +509,72 @@ __device__ __forceinline__ void score_table(const KParams &p, const Regions<Word
     }
 }
 
+// The scores of the exact selection from the level's own rows of counts, which score_table left:
+// E is read as it stands, T summed from the rows of A2 of the images as there. (With passes over
+// 2 W popcounts per column, 20 pairs of 500-1,000 vertices at K = 256 and costs of 700-3,001,
+// where nearly every level comes here, took 378 ms; 86 ms so.)
+template <int W, typename Word, bool FOLD>
+__device__ __forceinline__ void score_counts(const KParams &p, const Regions<Word> &R,
+                                             const LevelView<Word> &V, int n2, int anchor, int sh,
+                                             int32_t *hrow)
+{
+    constexpr int WBY = (int)sizeof(Word);
+    const int lane = threadIdx.x & 31;
+    const int N2S = p.lay.n2s;
+    const int c_eins = p.cost.eins, c_edel = p.cost.edel;
+    const uint8_t *a2b = (const uint8_t *)R.a2t, *imb = (const uint8_t *)V.imgw;
+    const int64_t NA = p.lay.rsize[RG_A2T], NE = p.lay.rsize[RG_ET0];
+    for (int s = V.s_lo; s < V.s_hi; ++s) {
+        for (int c0 = 8 * lane; c0 - 8 * lane < V.stride; c0 += 256) {   // the whole warp
+            const bool on = c0 < V.stride;
+            const int wrow = (c0 / (8 * WBY)) * N2S, by = (c0 >> 3) % WBY;
+            const bool in = c0 < 8 * WBY * W;   // (columns past the last word: no bits)
+            uint2 e = make_uint2(0u, 0u);
+            if (on) e = FG_AT((const uint2 *)V.et, ((int64_t)s * N2S + c0) >> 3, NE >> 3);
+            uint32_t tt[2] = {0u, 0u};
+            int np = 0;   // images of v_i's prior neighbours
+            for (int q0 = 0; q0 < V.deg; q0 += 32) {
+                int u = 0xffff;
+                if (q0 + lane < V.deg) {
+                    const int v = FG_AT(R.nbr, V.n0 + q0 + lane, FG_N(int32_t, p.lay.rsize[RG_NBR])) & 0xffff;
+                    u = FG_AT(V.map, (int64_t)s * V.mt + v, FG_N(uint16_t, p.lay.rsize[RG_MAP0]));
+                }
+                unsigned m = __ballot_sync(0xffffffffu, u != 0xffff);
+                np += __popc(m);
+                for (; m; m &= m - 1u) {
+                    const int img = __shfl_sync(0xffffffffu, u, __ffs((int)m) - 1);
+                    const uint32_t a = in ? (uint32_t)FG_AT(a2b, (int64_t)(wrow + img) * WBY + by, NA) : 0u;
+                    tt[0] += nibble_bytes(a);
+                    tt[1] += nibble_bytes(a >> 4);
+                }
+            }
+            if (!on) continue;
+            const int base = FG_AT(R.sbase, s - V.cs0, FG_N(int32_t, p.lay.rsize[RG_SBASE])) - anchor +
+                             (FOLD ? 0 : c_edel * np);
+            uint32_t um = c0 < n2 ? (uint32_t)FG_AT(imb, (int64_t)(s - V.ioff) * W * WBY + (c0 >> 3), V.nimg * WBY) : 0u;
+            if (c0 + 8 > n2 + 1) um |= c0 > n2 ? 0xffu : 0xffu << (n2 + 1 - c0);
+            uint32_t v4[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int4 cr = FG_AT((const int4 *)V.crow, (c0 >> 2) + h, N2S >> 2);
+                const int cw[4] = {cr.x, cr.y, cr.z, cr.w};
+                const uint32_t eh = h ? e.y : e.x;
+                const uint32_t f = FOLD ? eh + (uint32_t)np * 0x01010101u - 2u * tt[h] : eh - tt[h];
+                v4[h] = 0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    int d = base + cw[u] + c_eins * (int)((f >> (8 * u)) & 0xffu);
+                    if (!FOLD) d -= c_edel * (int)((tt[h] >> (8 * u)) & 0xffu);
+                    const int v = (um >> (4 * h + u)) & 1u ? kScoreMax : exact_byte(d, sh);
+                    if (v < kScoreMax) atomicAdd(&FG_AT(hrow, v, kBuckets), 1);
+                    v4[h] |= (uint32_t)v << (8 * u);
+                }
+            }
+            FG_AT((uint2 *)R.score, ((int64_t)(s - V.cs0) * V.stride + c0) >> 3, FG_N(uint2, p.lay.rsize[RG_SCORE])) = make_uint2(v4[0], v4[1]);
+        }
+    }
+}
+
 // Scores this warp's nodes again for the exact selection (the node vectors are in place). A warp
 // without nodes must not enter the scoring, which reads a column's tables before its first node:
 // the CTA may have none at all, and then no list of columns. (The test stands here and not in
@@ -514,7 +589,10 @@ __device__ __noinline__ void score_exact(const KParams &p, const Regions<Word> &
     for (int b = lane; b < kBuckets; b += 32) FG_AT(hrow, b, kBuckets) = 0;
     __syncwarp();
     if (V.s_lo >= V.s_hi) return;
-    if (p.cost.eins == p.cost.edel)
+    if (W >= 8 && V.et) {
+        if (p.cost.eins == p.cost.edel) score_counts<W, Word, true>(p, R, V, n2, anchor, sh, hrow);
+        else score_counts<W, Word, false>(p, R, V, n2, anchor, sh, hrow);
+    } else if (p.cost.eins == p.cost.edel)
         score_nodes<W, Word, BK, true, true>(p, R, V, B, n2, nw, V.s_lo, V.s_hi - V.s_lo, anchor, sh, hrow);
     else
         score_nodes<W, Word, BK, false, true>(p, R, V, B, n2, nw, V.s_lo, V.s_hi - V.s_lo, anchor, sh, hrow);
@@ -730,60 +808,157 @@ __device__ __forceinline__ int kept_code(const KParams &p, const Regions<Word> &
     return ((V.cs0 + (int)row) << kSelShift) | j;
 }
 
-// Exact selection, used when the kept set reaches past the histogram window: the level is
-// scored again over coarser, then finer PED windows until the K-th PED is known exactly, the
-// kept candidates are compacted stably and ordered by (PED, enumeration order).
-// thr >= 0: offset of the K-th PED from `anchor`, with `below` successors below it.
+// Region pointers of a team from a region -> base address function.
+template <typename Word, typename F>
+__device__ __forceinline__ Regions<Word> make_regions(F base)
+{
+    Regions<Word> R;
+    R.hist = (int32_t *)base(RG_HIST);
+    R.alpha2 = (int32_t *)base(RG_ALPHA2);
+    R.crow = (int32_t *)base(RG_CROW);
+    R.a2t = (Word *)base(RG_A2T);
+    R.l2t = (Word *)base(RG_L2T);
+    R.sbase = (int32_t *)base(RG_SBASE);
+    R.ped0 = (int32_t *)base(RG_PED0);
+    R.ped1 = (int32_t *)base(RG_PED1);
+    R.sel = (int32_t *)base(RG_SEL);
+    R.selped = (int32_t *)base(RG_SELPED);
+    R.klist = (int32_t *)base(RG_KLIST);
+    R.kped = (int32_t *)base(RG_KPED);
+    R.noff = (int32_t *)base(RG_NOFF);
+    R.nbr = (int32_t *)base(RG_NBR);
+    R.img0 = (Word *)base(RG_IMG0);
+    R.img1 = (Word *)base(RG_IMG1);
+    R.P = (Word *)base(RG_P);
+    R.PL = (Word *)base(RG_PL);
+    R.score = base(RG_SCORE);
+    R.et0 = base(RG_ET0);
+    R.et1 = base(RG_ET1);
+    R.chist = (int32_t *)base(RG_CHIST);
+    R.map0 = base(RG_MAP0);
+    R.map1 = base(RG_MAP1);
+    R.imgl = (Word *)base(RG_IMGL);
+    return R;
+}
+
+// The regions that every layout keeps in shared memory: histogram rows, active columns and
+// their records, and the used-by-all mask. Taken from the shared window directly, their accesses (the
+// histogram's increments above all) need no generic addressing.
+template <typename Word>
+__device__ __forceinline__ void smem_regions(const KParams &p, Regions<Word> &R, uint8_t *smem)
+{
+    R.hist = (int32_t *)(smem + p.lay.off[RG_HIST]);
+    R.act = (uint16_t *)(smem + p.lay.off[RG_ACT]);
+    R.allm = (uint32_t *)(smem + p.lay.off[RG_ALL]);
+    R.rec = smem + p.lay.off[RG_REC];
+}
+
+// A team's regions from the layout alone: what the kernels below build, with every base chosen
+// by the layout's masks.
+template <typename Word, bool CL>
+__device__ __forceinline__ Regions<Word> team_regions(const KParams &p)
+{
+    extern __shared__ __align__(16) uint8_t smem[];
+    const unsigned team = CL ? blockIdx.x / cluster_size() : blockIdx.x;
+    uint8_t *gs = p.gscratch + (int64_t)team * p.lay.slice_bytes;
+    uint8_t *gc = CL ? gs + p.lay.cta_off + (int64_t)cluster_rank() * p.lay.cta_bytes : gs;
+    Regions<Word> R = make_regions<Word>([&](int r) -> uint8_t * {
+        if ((p.lay.smem_mask >> r) & 1u) return smem + p.lay.off[r];
+        return (CL && ((p.lay.cta_mask >> r) & 1u) ? gc : gs) + p.lay.off[r];
+    });
+    smem_regions(p, R, smem);
+    return R;
+}
+
+// What the exact selection's functions know of level i (L nodes, nact columns in rows of `stride`
+// bytes). They build the team's regions and the warp's view of the level anew: handed over by
+// reference, both would live in the caller's local memory.
+struct ExactLevel {
+    int i, L, nact, stride, B, n2, nw;
+    bool table;   // rows of neighbour counts are kept
+};
+
+template <int W, typename Word, bool CL>
+__device__ __forceinline__ LevelView<Word> exact_view(const KParams &p, const Regions<Word> &R,
+                                                      const Team<CL> &tm, const ExactLevel &x)
+{
+    LevelView<Word> V;
+    const bool odd = x.i & 1;   // the beam buffers alternate
+    V.cs0 = CL ? (int)((int64_t)(tm.warp - (int)(threadIdx.x >> 5)) * x.L / tm.NW) : 0;
+    V.ioff = V.cs0;
+    V.imgw = CL ? R.imgl : odd ? R.img1 : R.img0;
+    V.nimg = FG_N(Word, p.lay.rsize[CL ? RG_IMGL : RG_IMG0]);
+    V.crow = R.crow + (odd ? p.lay.n2s : 0);
+    V.s_lo = (int)((int64_t)tm.warp * x.L / tm.NW);
+    V.s_hi = (int)((int64_t)(tm.warp + 1) * x.L / tm.NW);
+    V.nact = x.nact;
+    V.stride = x.stride;
+    if (W >= 8) {
+        V.et = x.table ? (odd ? R.et0 : R.et1) : nullptr;
+        V.map = (const uint16_t *)(odd ? R.map1 : R.map0);
+        V.mt = p.lay.mrow / (int64_t)sizeof(uint16_t);
+        V.n0 = FG_AT(R.noff, x.i, FG_N(int32_t, p.lay.rsize[RG_NOFF]));
+        V.deg = FG_AT(R.noff, x.i + 1, FG_N(int32_t, p.lay.rsize[RG_NOFF])) - V.n0;
+    }
+    return V;
+}
+
+// Exact selection, first part, for a K-th PED past the histogram window or below a guessed
+// anchor: the level is scored again over coarser, then finer PED windows until the K-th PED is
+// known. Returns the score byte of the K-th PED, the successors below it, and what added to a byte
+// gives its PED (byte 0: below the last window). The bytes and the histogram rows are those of
+// the last pass.
 template <int W, typename Word, int BK, bool CL>
-__device__ __noinline__ void select_exact(const KParams &p, const Regions<Word> &R,
-                                          const LevelView<Word> &V, int B, int n2, int nw,
-                                          int newL, int anchor, int thr, int below)
+__device__ __noinline__ int4 rescore_exact(const KParams &p, const ExactLevel x, int newL, int anchor)
 {
     const Team<CL> tm;
-    const int tid = tm.tid, T = tm.T, lane = threadIdx.x & 31;
+    const Regions<Word> R = team_regions<Word, CL>(p);
+    const LevelView<Word> V = exact_view<W, Word, CL>(p, R, tm, x);
     const int nwl = (int)blockDim.x >> 5, lw = (int)threadIdx.x >> 5;
     int32_t *hrow = R.hist + lw * kBuckets;
     const int32_t *htot = R.hist + nwl * kBuckets;
+    // windows of 127 buckets, each 64 times as wide as the one before, until one holds the K-th
+    // PED (PEDs are below 2^31, so a bucket width of 2^30 does); then 64 buckets of 1/64 the
+    // width inside the bucket found
+    int sh = 0, pre = 0, thr = 0, below = 0, first;
+    bool down = false;
+    for (int pass = 0; pass < 12; ++pass) {   // up to 30, then to 0
+        sh += down ? -6 : 6;
+        tm.sync();
+        score_exact<W, Word, BK>(p, R, V, x.B, x.n2, x.nw, anchor, sh, hrow);
+        prefix_buckets<CL>(p, R, tm);
+        // (the last pass counts the successors below its window as well)
+        find_threshold(p, htot, sh > 0 ? newL - pre : newL, thr, below, first);
+        if (sh == 0) break;
+        if (thr < kScoreMax) {
+            down = true;
+            pre += below;
+            anchor += thr << sh;
+        }
+    }
+    return make_int4(thr, below, anchor - 1, 0);
+}
+
+// Exact selection, second part: entries [kbeg, kbeg + kcnt) of the kept lists hold this warp's
+// compacted children (index and score byte); their codes and PEDs follow, and the team orders
+// all newL by (PED, enumeration order). low: byte 0 stands for any PED below.
+template <int W, typename Word, int BK, bool CL>
+__device__ __noinline__ void order_exact(const KParams &p, const ExactLevel x, int newL, int anchor,
+                                         bool low, int kbeg, int kcnt)
+{
+    const Team<CL> tm;
+    const Regions<Word> R = team_regions<Word, CL>(p);
+    const LevelView<Word> V = exact_view<W, Word, CL>(p, R, tm, x);
+    const int tid = tm.tid, T = tm.T, lane = threadIdx.x & 31;
 #define NKP FG_N(int32_t, p.lay.rsize[RG_KPED])
 #define NKL FG_N(int32_t, p.lay.rsize[RG_KLIST])
 #define NSE FG_N(int32_t, p.lay.rsize[RG_SEL])
 #define NSP FG_N(int32_t, p.lay.rsize[RG_SELPED])
-    if (thr < 0) {
-        // windows of 127 buckets, each 64 times as wide as the one before, until one holds the
-        // K-th PED (PEDs are below 2^31, so a bucket width of 2^30 does); then 64 buckets of
-        // 1/64 the width inside the bucket found
-        int sh = 0, pre = 0, first;
-        bool down = false;
-        for (int pass = 0; pass < 12 && !(down && sh == 0); ++pass) {   // up to 30, then to 0
-            sh += down ? -6 : 6;
-            tm.sync();
-            score_exact<W, Word, BK>(p, R, V, B, n2, nw, anchor, sh, hrow);
-            prefix_buckets<CL>(p, R, tm);
-            find_threshold(p, htot, newL - pre, thr, below, first);
-            if (thr < kScoreMax) {
-                down = true;
-                pre += below;
-                anchor += thr << sh;
-            }
-        }
-        below = pre;
-    } else {
-        anchor += thr;
-    }
-    const int q = newL - below;
-    tm.sync();
-    score_exact<W, Word, BK>(p, R, V, B, n2, nw, anchor, -1, hrow);
-    prefix_buckets<CL>(p, R, tm);
-    {
-        const int lt = FG_AT(hrow, 0, kBuckets), eq = FG_AT(hrow, 1, kBuckets);
-        const int kbeg = lt + min(q, eq);
-        const int kcnt = compact_kept<Word>(p, R, V, 1, q, kbeg, eq);
-        __syncwarp();
-        for (int x = kbeg + lane; x < kbeg + kcnt; x += 32) {
-            const int code = kept_code<Word>(p, R, V, FG_AT(R.klist, x, NKL));
-            FG_AT(R.klist, x, NKL) = code;
-            FG_AT(R.kped, x, NKP) = succ_ped<W, Word>(p, R, V, B, code >> kSelShift, code & ((1 << kSelShift) - 1));
-        }
+    for (int a = kbeg + lane; a < kbeg + kcnt; a += 32) {
+        const int code = kept_code<Word>(p, R, V, FG_AT(R.klist, a, NKL)), v = FG_AT(R.kped, a, NKP);
+        FG_AT(R.klist, a, NKL) = code;
+        FG_AT(R.kped, a, NKP) = low && v == 0 ? succ_ped<W, Word>(p, R, V, x.B, code >> kSelShift, code & ((1 << kSelShift) - 1))
+                                              : anchor + v;
     }
     tm.sync();
     // order by (PED, enumeration order); klist is in enumeration order and its codes are
@@ -1309,11 +1484,13 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
         find_threshold(p, htot, newL, thr, below, first);
         const bool fits = A == A0 || first > 0;   // nothing below the anchor
         rise = A - A0 + (first < kScoreMax ? first : kScoreMax);
-        if (fits && thr < kScoreMax && thr - first < hwin - 1) {
-            // kept = every successor below the threshold bucket and the first q in it. Each
-            // warp compacts its kept successors in enumeration order, then places them at
-            // their rank in (PED, parent slot, j) order: position = #(smaller PED) +
-            // #(equal PED earlier); lane b answers for bucket first + b.
+        // kept = every successor below the threshold bucket and the first q in it. Each warp
+        // compacts its kept successors in enumeration order, then places them at their rank in
+        // (PED, parent slot, j) order: position = #(smaller PED) + #(equal PED earlier); lane b
+        // answers for bucket first + b. Kept sets past the window or over too many buckets go
+        // through the exact selection instead.
+        const bool known = fits && thr < kScoreMax;
+        if (known && thr - first < hwin - 1) {
             const int q = newL - below;
             const bool in = first + lane <= thr;
             int incl = in ? FG_AT(htot, first + lane, kBuckets) : 0;
@@ -1355,8 +1532,23 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
             }
             PHASE_MARK(9);
         } else {
-            const bool known = fits && thr < kScoreMax;
-            select_exact<W, Word, BK, CL>(p, R, V, B, n2, nw, newL, fits ? A : A0, known ? thr : -1, below);
+            const ExactLevel x = {i, L, nact, stride, B, n2, nw, W >= 8 && table};
+            int anchor = A;
+            if (!known) {
+                const int4 found = rescore_exact<W, Word, BK, CL>(p, x, newL, fits ? A : A0);
+                thr = found.x;
+                below = found.y;
+                anchor = found.z;
+            }
+            const int q = newL - below;
+            int lt = 0;   // successors of earlier warps in the buckets below thr
+            for (int b = lane; b < thr; b += 32) lt += FG_AT(hrow, b, kBuckets);
+            lt = warp_sum(lt);
+            const int eq = FG_AT(hrow, thr, kBuckets);
+            const int kbeg = lt + min(q, eq);
+            const int kcnt = compact_kept<Word>(p, R, V, thr, q, kbeg, eq);
+            __syncwarp();
+            order_exact<W, Word, BK, CL>(p, x, newL, anchor, !known, kbeg, kcnt);
             PHASE_MARK(10);
         }
         tm.sync();
@@ -1532,51 +1724,6 @@ __device__ __forceinline__ void solve_pair(const KParams &p, const Regions<Word>
 #undef NMAPT
 #undef NMAP16
 #undef NIMGW
-}
-
-// Region pointers of a team from a region -> base address function.
-template <typename Word, typename F>
-__device__ __forceinline__ Regions<Word> make_regions(F base)
-{
-    Regions<Word> R;
-    R.hist = (int32_t *)base(RG_HIST);
-    R.alpha2 = (int32_t *)base(RG_ALPHA2);
-    R.crow = (int32_t *)base(RG_CROW);
-    R.a2t = (Word *)base(RG_A2T);
-    R.l2t = (Word *)base(RG_L2T);
-    R.sbase = (int32_t *)base(RG_SBASE);
-    R.ped0 = (int32_t *)base(RG_PED0);
-    R.ped1 = (int32_t *)base(RG_PED1);
-    R.sel = (int32_t *)base(RG_SEL);
-    R.selped = (int32_t *)base(RG_SELPED);
-    R.klist = (int32_t *)base(RG_KLIST);
-    R.kped = (int32_t *)base(RG_KPED);
-    R.noff = (int32_t *)base(RG_NOFF);
-    R.nbr = (int32_t *)base(RG_NBR);
-    R.img0 = (Word *)base(RG_IMG0);
-    R.img1 = (Word *)base(RG_IMG1);
-    R.P = (Word *)base(RG_P);
-    R.PL = (Word *)base(RG_PL);
-    R.score = base(RG_SCORE);
-    R.et0 = base(RG_ET0);
-    R.et1 = base(RG_ET1);
-    R.chist = (int32_t *)base(RG_CHIST);
-    R.map0 = base(RG_MAP0);
-    R.map1 = base(RG_MAP1);
-    R.imgl = (Word *)base(RG_IMGL);
-    return R;
-}
-
-// The regions that every layout keeps in shared memory: histogram rows, active columns and
-// their records, and the used-by-all mask. Taken from the shared window directly, their accesses (the
-// histogram's increments above all) need no generic addressing.
-template <typename Word>
-__device__ __forceinline__ void smem_regions(const KParams &p, Regions<Word> &R, uint8_t *smem)
-{
-    R.hist = (int32_t *)(smem + p.lay.off[RG_HIST]);
-    R.act = (uint16_t *)(smem + p.lay.off[RG_ACT]);
-    R.allm = (uint32_t *)(smem + p.lay.off[RG_ALL]);
-    R.rec = smem + p.lay.off[RG_REC];
 }
 
 // SM: every region but the neighbour lists and the vertex maps lives in shared memory (addresses then stay in the

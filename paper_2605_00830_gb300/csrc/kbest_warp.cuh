@@ -37,7 +37,7 @@
 // matrix, K = 20: 1.28 -> 1.19 ms. (One pair from host memory: 302 -> 296 us; a batch that small
 // takes a CTA per pair, 209 us. team_beats_warps in fastged_runtime.cu says where the line lies.)
 // Registers are capped at 96 by the launch bounds; the instances with 0 and 2 label planes spill
-// 16-36 bytes for it.
+// 20-40 bytes for it.
 #pragma once
 #include "kbest_impl.cuh"
 
@@ -151,8 +151,8 @@ struct WarpLevel {
 };
 
 // Scores every successor of level i. MODE 0: bytes and counts of the offsets from A; returns the
-// successors of the level. MODE 1 (selection past the window): with sh >= 0 the offsets from A
-// in units of 2^sh, PEDs below A left out; sh < 0 marks 0 = below A, 1 = at A, 127 = above.
+// successors of the level. MODE 1 (selection past the window): with sh > 0 the offsets from A
+// in units of 2^sh, PEDs below A left out; sh == 0 gives 0 below A and 1 + the offset from A on.
 // MODE 2 (variant B's last level): no bytes; the lane's least (total, PED, code) of the
 // completed successors goes to key and code.
 // FOLD: insertion and deletion of an edge cost the same, so the two implied-edge terms are
@@ -293,8 +293,8 @@ __device__ __forceinline__ int eval_level(const KParams &p,
                         const int d = dd[u];
                         int v;
                         if (MODE == 0) v = min(d, kScoreMax);
-                        else if (sh >= 0) v = d < 0 ? kScoreMax : min(d >> sh, kScoreMax);
-                        else v = d < 0 ? 0 : d == 0 ? 1 : kScoreMax;
+                        else if (sh > 0) v = d < 0 ? kScoreMax : min(d >> sh, kScoreMax);
+                        else v = d < 0 ? 0 : min(d + 1, kScoreMax);
                         if (us[u]) v = kScoreMax;
                         dd[u] = v;
                         atomicAdd(&FG_AT(hist, v, kBuckets), 1);   // [127] is not read
@@ -329,8 +329,11 @@ __device__ __forceinline__ int warp_code(const KParams &p, const WarpRegs<Word, 
     return (s << 8) | (bit ? popcw((Word)(bit - 1)) : n2);
 }
 
-// Exact selection: the kept PEDs reach past the histogram window (which starts at A).
-// thr >= 0: offset of the K-th PED, with `below` successors below it.
+// Exact selection: the kept PEDs reach past the histogram window (which starts at A), or over
+// too many of its buckets. thr >= 0: offset of the K-th PED, with `below` successors below it;
+// the score bytes then hold the kept PEDs already. Otherwise the level is scored again, two or
+// four times, and the bytes of the last pass select (no further pass marks the kept ones: 5,000
+// molecule pairs with costs of 700-3,001, where nearly every level comes here, 9.0 -> 8.4 ms).
 template <typename Word, int BK, bool FOLD>
 __device__ __noinline__ void select_exact_warp(const KParams &p,
                                                const WarpRegs<Word, (BK == 8 ? kMaxB : BK)> R,
@@ -344,73 +347,78 @@ __device__ __noinline__ void select_exact_warp(const KParams &p,
     int32_t *hist = R.hist(wl);
     unsigned long long key = 0;
     int code = 0;
+    const bool known = thr >= 0;
     int anchor = A;
-    auto score_at = [&](int sh) {
-        for (int b = lane; b < kBuckets; b += 32) FG_AT(hist, b, kBuckets) = 0;
-        __syncwarp();
-        eval_level<Word, BK, FOLD, 1>(p, R, lv, anchor, sh, key, code);
-    };
-    if (thr < 0) {
+    if (!known) {
         // windows 64 times as wide as the one before until one holds the K-th PED (PEDs are
         // below 2^16 here), then 64 buckets of 1/64 the width inside the bucket found
         int sh = 0, pre = 0, first;
         bool down = false;
-        for (int pass = 0; pass < 12 && !(down && sh == 0); ++pass) {
+        for (int pass = 0; pass < 12; ++pass) {
             sh += down ? -6 : 6;
-            score_at(sh);
-            find_threshold(p, hist, newL - pre, thr, below, first);
+            for (int b = lane; b < kBuckets; b += 32) FG_AT(hist, b, kBuckets) = 0;
             __syncwarp();
+            eval_level<Word, BK, FOLD, 1>(p, R, lv, anchor, sh, key, code);
+            // (the last pass counts the successors below its window as well)
+            find_threshold(p, hist, sh > 0 ? newL - pre : newL, thr, below, first);
+            __syncwarp();
+            if (sh == 0) break;
             if (thr < kScoreMax) {
                 down = true;
                 pre += below;
                 anchor += thr << sh;
             }
         }
-        below = pre;
-    } else {
-        anchor += thr;
     }
-    score_at(-1);
     uint32_t *klist = R.klist(wl);
-    compact_bytes(p, R.score(wl), NSC, 0, lv.L * row, 1, newL - below, 0, 0, newL,
-                  [&](int at, int idx, int) { FG_AT(klist, at, FG_N(uint32_t, wl.size[WR_KLIST])) = (uint32_t)idx; });
+    compact_bytes(p, R.score(wl), NSC, 0, lv.L * row, thr, newL - below, 0, 0, newL,
+                  [&](int at, int idx, int v) {
+                      FG_AT(klist, at, FG_N(uint32_t, wl.size[WR_KLIST])) = ((uint32_t)v << 16) | (uint32_t)idx;
+                  });
     __syncwarp();
-    // PED of every kept child, from the definition; selped holds it in enumeration order
+    // code and PED of every kept child, in enumeration order: the PED from its byte, or from the
+    // definition for those below the last window
     for (int x = lane; x < newL; x += 32) {
-        const int cc = warp_code<Word, NPL>(p, R, (int)FG_AT(klist, x, FG_N(uint32_t, wl.size[WR_KLIST])), row, inv, lv.n2);
-        const int s = cc >> 8, j = cc & 0xff;
-        const TgtRec<Word, NPL> t = FG_AT(R.tgt(wl), j, (int64_t)wl.size[WR_TGT] / (int64_t)sizeof(TgtRec<Word, NPL>));
-        Word P = (Word)0, z = (Word)0;
-        int dcnt = 0;
-        for (int q = 0; q < lv.deg; ++q) {
-            const int e = FG_AT(R.nbr(wl), lv.n0 + q, FG_N(int32_t, wl.size[WR_NBR]));
-            const uint8_t ph = FG_AT(R.mapc(wl), (int64_t)s * lv.mrow + (e & 0xffff), wl.size[WR_MAP0]);
-            if (ph == 0xff) { ++dcnt; continue; }
-            const Word pb = (Word)1 << ph;
-            P |= pb;
-            for (int b = 0; b < B; ++b)
-                z |= (((e >> (16 + b)) & 1 ? pb : (Word)0) ^ rec_plane(t, b)) & pb;
+        const uint32_t kv = FG_AT(klist, x, FG_N(uint32_t, wl.size[WR_KLIST]));
+        const int idx = (int)(kv & 0xffffu), v = (int)(kv >> 16);
+        const int cc = warp_code<Word, NPL>(p, R, idx, row, inv, lv.n2);
+        int ped = known ? A + v : anchor + v - 1;
+        if (!known && v == 0) {
+            const int s = cc >> 8, j = cc & 0xff;
+            const TgtRec<Word, NPL> t = FG_AT(R.tgt(wl), j, (int64_t)wl.size[WR_TGT] / (int64_t)sizeof(TgtRec<Word, NPL>));
+            Word P = (Word)0, z = (Word)0;
+            int dcnt = 0;
+            for (int q = 0; q < lv.deg; ++q) {
+                const int e = FG_AT(R.nbr(wl), lv.n0 + q, FG_N(int32_t, wl.size[WR_NBR]));
+                const uint8_t ph = FG_AT(R.mapc(wl), (int64_t)s * lv.mrow + (e & 0xffff), wl.size[WR_MAP0]);
+                if (ph == 0xff) { ++dcnt; continue; }
+                const Word pb = (Word)1 << ph;
+                P |= pb;
+                for (int b = 0; b < B; ++b)
+                    z |= (((e >> (16 + b)) & 1 ? pb : (Word)0) ^ rec_plane(t, b)) & pb;
+            }
+            const Word im = FG_AT(R.imgc(wl), s, FG_N(Word, wl.size[WR_IMG0])), ai = t.a2 & im;
+            ped = FG_AT(R.pedc(wl), s, FG_N(int32_t, wl.size[WR_PED0])) + p.cost.edel * dcnt +
+                  FG_AT(R.rec(wl), idx - s * row, NRC).crow + p.cost.eins * popcw((Word)(ai & ~P)) +
+                  p.cost.edel * popcw((Word)(P & ~t.a2)) + p.cost.esub * popcw((Word)(t.a2 & z));
         }
-        const Word im = FG_AT(R.imgc(wl), s, FG_N(Word, wl.size[WR_IMG0])), ai = t.a2 & im;
-        const int crow = FG_AT(R.rec(wl), (int)FG_AT(klist, x, FG_N(uint32_t, wl.size[WR_KLIST])) - s * row, NRC).crow;
         FG_AT(klist, x, FG_N(uint32_t, wl.size[WR_KLIST])) = (uint32_t)cc;
-        FG_AT(R.selped(wl), x, FG_N(int32_t, wl.size[WR_SELPED])) =
-            FG_AT(R.pedc(wl), s, FG_N(int32_t, wl.size[WR_PED0])) + p.cost.edel * dcnt + crow +
-            p.cost.eins * popcw((Word)(ai & ~P)) + p.cost.edel * popcw((Word)(P & ~t.a2)) +
-            p.cost.esub * popcw((Word)(t.a2 & z));
+        FG_AT(R.selped(wl), x, FG_N(int32_t, wl.size[WR_SELPED])) = ped;
     }
     __syncwarp();
-    // rank by (PED, enumeration order); at most kWarpChunks children per lane
+    // rank by (PED, enumeration order); at most kWarpChunks children per lane, and PEDs below 2^16
+    // beside seven bits of the order
     int rk[kWarpChunks], pd[kWarpChunks];
 #pragma unroll
     for (int ch = 0; ch < kWarpChunks; ++ch) {
         const int x = 32 * ch + lane;
         rk[ch] = 0;
         pd[ch] = x < newL ? FG_AT(R.selped(wl), x, FG_N(int32_t, wl.size[WR_SELPED])) : 0;
-        for (int y = 0; x < newL && y < newL; ++y) {
-            const int py = FG_AT(R.selped(wl), y, FG_N(int32_t, wl.size[WR_SELPED]));
-            rk[ch] += py < pd[ch] || (py == pd[ch] && y < x);
-        }
+    }
+    for (int y = 0; y < newL; ++y) {
+        const int ky = FG_AT(R.selped(wl), y, FG_N(int32_t, wl.size[WR_SELPED])) << 7 | y;
+#pragma unroll
+        for (int ch = 0; ch < kWarpChunks; ++ch) rk[ch] += ky < (pd[ch] << 7 | (32 * ch + lane));
     }
     __syncwarp();
 #pragma unroll
